@@ -405,37 +405,118 @@ __global__ void __launch_bounds__(256, FEW ? 2 : 4) k_dual(SweepArgs a) {
     }
 }
 
+// Conditional additions of up to seven set dual bits, bits 0..n-1 of m.  A bit
+// test and a predicated add per entry kept the ALU pipe of the primal step busy
+// (two cycles per warp for a test); written as one block of bit tests followed
+// by the adds, the tests of a block become one move of the word into the seven
+// predicate registers.  49 entries took 65 ALU-pipe instructions before and
+// take 17 (12 of them shifts and moves of the words).
+#define MRF_BT1(M) "and.b32 a0," M ",1;setp.ne.u32 p0,a0,0;"
+#define MRF_BT2(M) MRF_BT1(M) "and.b32 a1," M ",2;setp.ne.u32 p1,a1,0;"
+#define MRF_BT3(M) MRF_BT2(M) "and.b32 a2," M ",4;setp.ne.u32 p2,a2,0;"
+#define MRF_BT4(M) MRF_BT3(M) "and.b32 a3," M ",8;setp.ne.u32 p3,a3,0;"
+#define MRF_BT5(M) MRF_BT4(M) "and.b32 a4," M ",16;setp.ne.u32 p4,a4,0;"
+#define MRF_BT6(M) MRF_BT5(M) "and.b32 a5," M ",32;setp.ne.u32 p5,a5,0;"
+#define MRF_BT7(M) MRF_BT6(M) "and.b32 a6," M ",64;setp.ne.u32 p6,a6,0;"
+#define MRF_BR1 "@p0 add.f32 %0,%0,%2;"
+#define MRF_BR2 MRF_BR1 "@p1 add.f32 %0,%0,%3;"
+#define MRF_BR3 MRF_BR2 "@p2 add.f32 %0,%0,%4;"
+#define MRF_BR4 MRF_BR3 "@p3 add.f32 %0,%0,%5;"
+#define MRF_BR5 MRF_BR4 "@p4 add.f32 %0,%0,%6;"
+#define MRF_BR6 MRF_BR5 "@p5 add.f32 %0,%0,%7;"
+#define MRF_BR7 MRF_BR6 "@p6 add.f32 %0,%0,%8;"
+#define MRF_BE1 "@p0 add.f32 %0,%0,%8;"
+#define MRF_BE2 MRF_BE1 "@p1 add.f32 %1,%1,%9;"
+#define MRF_BE3 MRF_BE2 "@p2 add.f32 %2,%2,%10;"
+#define MRF_BE4 MRF_BE3 "@p3 add.f32 %3,%3,%11;"
+#define MRF_BE5 MRF_BE4 "@p4 add.f32 %4,%4,%12;"
+#define MRF_BE6 MRF_BE5 "@p5 add.f32 %5,%5,%13;"
+#define MRF_BE7 MRF_BE6 "@p6 add.f32 %6,%6,%14;"
+#define MRF_BITS_REGS "{.reg .pred p0,p1,p2,p3,p4,p5,p6;.reg .b32 a0,a1,a2,a3,a4,a5,a6;"
+#define MRF_BITS_ROW(n)                                                                                        \
+    if constexpr (N == n)                                                                                      \
+        asm(MRF_BITS_REGS MRF_BT##n("%1") MRF_BR##n "}"                                                        \
+            : "+f"(acc)                                                                                        \
+            : "r"(m), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(t[4]), "f"(t[5]), "f"(t[6]))
+#define MRF_BITS_EACH(n)                                                                                       \
+    if constexpr (N == n)                                                                                      \
+        asm(MRF_BITS_REGS MRF_BT##n("%7") MRF_BE##n "}"                                                        \
+            : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]), "+f"(r[6])               \
+            : "r"(m), "f"(t[0]), "f"(t[1]), "f"(t[2]), "f"(t[3]), "f"(t[4]), "f"(t[5]), "f"(t[6]))
+
+// acc += t[0..N-1] of the set bits, in order.
+template <int N>
+__device__ __forceinline__ void add_bits_row(uint32_t m, const float (&t)[7], float& acc) {
+    MRF_BITS_ROW(1); MRF_BITS_ROW(2); MRF_BITS_ROW(3); MRF_BITS_ROW(4); MRF_BITS_ROW(5); MRF_BITS_ROW(6); MRF_BITS_ROW(7);
+}
+
+// acc[i] += t[i] for every set bit i < N.
+template <int N>
+__device__ __forceinline__ void add_bits_each(uint32_t m, const float (&t)[7], float* acc) {
+    float r[7];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) r[i] = i < N ? acc[i] : 0.0f;
+    MRF_BITS_EACH(1); MRF_BITS_EACH(2); MRF_BITS_EACH(3); MRF_BITS_EACH(4); MRF_BITS_EACH(5); MRF_BITS_EACH(6);
+    MRF_BITS_EACH(7);
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = r[i];
+}
+
+// Entries [K0, K0 + N) of one table row: the dual words' bits K0.. as the low bits of a word.
+template <int K0, int N, int W>
+__device__ __forceinline__ uint32_t entry_bits(const uint32_t (&bits)[W]) {
+    constexpr int g = K0 >> 5, sh = K0 & 31;
+    if constexpr (sh == 0) return bits[g];
+    else if constexpr (sh + N <= 32) return bits[g] >> sh;
+    else return __funnelshift_r(bits[g], bits[g + 1 < W ? g + 1 : g], sh);
+}
+
+// Entries K0 .. K1-1 of one table row (PIVOT: row label i, first column label
+// j0; DIAG: entries are labels), seven at a time.
+template <int L, int LAYOUT, int K0, int K1>
+__device__ __forceinline__ void add_span(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float (&tv)[Ent<L, LAYOUT>::MP],
+                                         int side, float (&acc)[L]) {
+    if constexpr (K0 < K1) {
+        using E = Ent<L, LAYOUT>;
+        constexpr int N = K1 - K0 < 7 ? K1 - K0 : 7;
+        const uint32_t m = entry_bits<K0, N, E::W>(bits);
+        float t[7];
+#pragma unroll
+        for (int i = 0; i < 7; ++i) t[i] = i < N ? (side == 0 ? tv[K0 + (i < N ? i : 0)] : fabsf(tv[K0 + (i < N ? i : 0)])) : 0.0f;
+        if (LAYOUT == MRF_LAYOUT_PIVOT && side == 0) add_bits_row<N>(m, t, acc[E::i(K0)]);
+        else add_bits_each<N>(m, t, acc + E::j(K0));
+        add_span<L, LAYOUT, K0 + N, K1>(bits, tv, side, acc);
+    }
+}
+
+template <int L, int LAYOUT, bool GLOBAL, int ROW>
+__device__ __forceinline__ void add_rows(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float4* __restrict__ t4,
+                                         float (&tv)[Ent<L, LAYOUT>::MP], int side, float (&acc)[L]) {
+    using E = Ent<L, LAYOUT>;
+    constexpr int R = LAYOUT == MRF_LAYOUT_PIVOT ? L - 1 : L;      // entries per table row
+    if constexpr (ROW * R < E::M) {
+        constexpr int q0 = (ROW * R + 3) / 4, q1 = ((ROW + 1) * R + 3) / 4;   // vectors not loaded by earlier rows
+#pragma unroll
+        for (int k4 = q0; k4 < q1; ++k4) {
+            const float4 q = GLOBAL ? __ldg(t4 + k4) : t4[k4];
+            tv[4 * k4] = q.x; tv[4 * k4 + 1] = q.y; tv[4 * k4 + 2] = q.z; tv[4 * k4 + 3] = q.w;
+        }
+        add_span<L, LAYOUT, ROW * R, (ROW + 1) * R>(bits, tv, side, acc);
+        add_rows<L, LAYOUT, GLOBAL, ROW + 1>(bits, t4, tv, side, acc);
+    }
+}
+
 // Accumulate the beta terms of edge e's set dual bits for one endpoint side
-// (tau row loaded as 16-byte vectors; beta1 = tau_signed, beta2 = |tau_signed|).
+// (tau row loaded as 16-byte vectors; beta1 = tau_signed, beta2 = |tau_signed|),
+// in entry order.
 // GLOBAL: the row is in global memory (read-only path); else in shared memory.
 template <int L, int LAYOUT, bool GLOBAL = true>
 __device__ __forceinline__ void add_side(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
                                          int side, float (&acc)[L]) {
-    using E = Ent<L, LAYOUT>;
     const float4* t4 = reinterpret_cast<const float4*>(tau_e);
-    if (side == 0) {
-#pragma unroll
-        for (int k4 = 0; k4 < E::MP / 4; ++k4) {
-            const float4 q = GLOBAL ? __ldg(t4 + k4) : t4[k4];
-            const float tv[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int k = 4 * k4 + u;
-                if (k < E::M && ((bits[k >> 5] >> (k & 31)) & 1u)) acc[E::i(k)] += tv[u];
-            }
-        }
-    } else {
-#pragma unroll
-        for (int k4 = 0; k4 < E::MP / 4; ++k4) {
-            const float4 q = GLOBAL ? __ldg(t4 + k4) : t4[k4];
-            const float tv[4] = {q.x, q.y, q.z, q.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int k = 4 * k4 + u;
-                if (k < E::M && ((bits[k >> 5] >> (k & 31)) & 1u)) acc[E::j(k)] += fabsf(tv[u]);
-            }
-        }
-    }
+    float tv[Ent<L, LAYOUT>::MP];
+    if (side == 0) add_rows<L, LAYOUT, GLOBAL, 0>(bits, t4, tv, 0, acc);
+    else add_rows<L, LAYOUT, GLOBAL, 0>(bits, t4, tv, 1, acc);
 }
 
 // Compensated (two-sum) flush of a float32 partial sum into a hi/lo pair, used
