@@ -19,6 +19,8 @@
 #pragma once
 #include "common.cuh"
 
+#include <algorithm>
+
 namespace mrfk {
 
 // ---------------------------------------------------------------------------- entry masks
@@ -247,6 +249,50 @@ __device__ __forceinline__ void dual_bits(uint32_t e, uint32_t c, int xs, int xt
 
 // ---------------------------------------------------------------------------- label draw
 
+// The uniform of the top 23 bits of a Philox word: (U + 1/2) 2^-23, exact in float32.
+__device__ __forceinline__ float uniform23(uint32_t word) {
+    return __uint_as_float(0x3F800000u | (word >> 9)) - 0x1.fffffep-1f;
+}
+
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0,%1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// First label a with u < cdf_a where the float32 inverse CDF below is sure to
+// agree, -1 otherwise.  The unnormalised sums c_a of the hardware's 2^x
+// (relative error 2^-22) are within 2e-6 s of the exact sums, and the CDF of
+// the full computation (expf, division, L <= 16 additions) within 3e-6 of the
+// exact one; so if every |c_a - u s| is at least 2^-16 s, both give the same
+// label, and no boundary is within the 1e-6 that draw_label counts.  Takes 7
+// instructions per label where the full computation takes 18; about one draw in
+// 4,000 (L = 8) falls back to it.  NaN and infinite fields always do.
+template <int L>
+__device__ __forceinline__ int draw_label_fast(const float (&F)[L], float u) {
+    constexpr float kLog2e = 1.4426950408889634f;
+    float mx = F[0];
+#pragma unroll
+    for (int a = 1; a < L; ++a) mx = fmaxf(mx, F[a]);
+    const float mb = mx * kLog2e;
+    float c[L], s = 0.0f;
+#pragma unroll
+    for (int a = 0; a < L; ++a) {
+        s += ex2_approx(fmaf(F[a], kLog2e, -mb));
+        c[a] = s;
+    }
+    const float us = u * s;
+    float closest = INFINITY;
+    int lab = 0;
+#pragma unroll
+    for (int a = 0; a < L; ++a) {
+        const float d = c[a] - us;
+        closest = fminf(closest, fabsf(d));
+        lab += d <= 0.0f ? 1 : 0;
+    }
+    return closest >= s * 0x1p-16f ? lab : -1;
+}
+
 // Draw x_v from exp(F)/Z by the inverse CDF with the 23-bit uniform u of
 // Philox phase `phase` (u is exact in float32); optionally record log p.
 // Counts draws within 1e-6 of a CDF boundary.
@@ -255,6 +301,11 @@ template <int L>
 __device__ __forceinline__ int draw_label(const float (&F)[L], uint32_t v, uint32_t c, uint32_t sweep,
                                           const RoundKeys& key, uint32_t phase, float* __restrict__ logp_out, Ctl* ctl,
                                           float* __restrict__ lp_drawn = nullptr) {
+    const float u = uniform23(draw_rk(v, sweep, c, phase, 0, key).x);
+    if (!logp_out && !lp_drawn) {
+        const int lab = draw_label_fast<L>(F, u);
+        if (lab >= 0) return lab;
+    }
     float mx = F[0];
 #pragma unroll
     for (int a = 1; a < L; ++a) mx = fmaxf(mx, F[a]);
@@ -271,8 +322,6 @@ __device__ __forceinline__ int draw_label(const float (&F)[L], uint32_t v, uint3
 #pragma unroll
         for (int a = 0; a < L; ++a) logp_out[a] = (F[a] - mx) - ls;
     }
-    const uint32_t U = draw_rk(v, sweep, c, phase, 0, key).x >> 9;
-    const float u = ((float)U + 0.5f) * (1.0f / 8388608.0f);
     float cdf = 0.0f;
     int lab = -1, last_pos = 0;
     bool near = false;
@@ -472,26 +521,29 @@ __device__ __forceinline__ uint32_t entry_bits(const uint32_t (&bits)[W]) {
 }
 
 // Entries K0 .. K1-1 of one table row (PIVOT: row label i, first column label
-// j0; DIAG: entries are labels), seven at a time.
-template <int L, int LAYOUT, int K0, int K1>
-__device__ __forceinline__ void add_span(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float (&tv)[Ent<L, LAYOUT>::MP],
-                                         int side, float (&acc)[L]) {
+// j0; DIAG: entries are labels), seven at a time, for CH chains.
+template <int L, int LAYOUT, int CH, int K0, int K1>
+__device__ __forceinline__ void add_span(const uint32_t (&bits)[CH][Ent<L, LAYOUT>::W],
+                                         const float (&tv)[Ent<L, LAYOUT>::MP], int side, float (&acc)[CH][L]) {
     if constexpr (K0 < K1) {
         using E = Ent<L, LAYOUT>;
         constexpr int N = K1 - K0 < 7 ? K1 - K0 : 7;
-        const uint32_t m = entry_bits<K0, N, E::W>(bits);
         float t[7];
 #pragma unroll
         for (int i = 0; i < 7; ++i) t[i] = i < N ? (side == 0 ? tv[K0 + (i < N ? i : 0)] : fabsf(tv[K0 + (i < N ? i : 0)])) : 0.0f;
-        if (LAYOUT == MRF_LAYOUT_PIVOT && side == 0) add_bits_row<N>(m, t, acc[E::i(K0)]);
-        else add_bits_each<N>(m, t, acc + E::j(K0));
-        add_span<L, LAYOUT, K0 + N, K1>(bits, tv, side, acc);
+#pragma unroll
+        for (int h = 0; h < CH; ++h) {
+            const uint32_t m = entry_bits<K0, N, E::W>(bits[h]);
+            if (LAYOUT == MRF_LAYOUT_PIVOT && side == 0) add_bits_row<N>(m, t, acc[h][E::i(K0)]);
+            else add_bits_each<N>(m, t, &acc[h][E::j(K0)]);
+        }
+        add_span<L, LAYOUT, CH, K0 + N, K1>(bits, tv, side, acc);
     }
 }
 
-template <int L, int LAYOUT, bool GLOBAL, int ROW>
-__device__ __forceinline__ void add_rows(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float4* __restrict__ t4,
-                                         float (&tv)[Ent<L, LAYOUT>::MP], int side, float (&acc)[L]) {
+template <int L, int LAYOUT, bool GLOBAL, int CH, int ROW>
+__device__ __forceinline__ void add_rows(const uint32_t (&bits)[CH][Ent<L, LAYOUT>::W], const float4* __restrict__ t4,
+                                         float (&tv)[Ent<L, LAYOUT>::MP], int side, float (&acc)[CH][L]) {
     using E = Ent<L, LAYOUT>;
     constexpr int R = LAYOUT == MRF_LAYOUT_PIVOT ? L - 1 : L;      // entries per table row
     if constexpr (ROW * R < E::M) {
@@ -501,22 +553,29 @@ __device__ __forceinline__ void add_rows(const uint32_t (&bits)[Ent<L, LAYOUT>::
             const float4 q = GLOBAL ? __ldg(t4 + k4) : t4[k4];
             tv[4 * k4] = q.x; tv[4 * k4 + 1] = q.y; tv[4 * k4 + 2] = q.z; tv[4 * k4 + 3] = q.w;
         }
-        add_span<L, LAYOUT, ROW * R, (ROW + 1) * R>(bits, tv, side, acc);
-        add_rows<L, LAYOUT, GLOBAL, ROW + 1>(bits, t4, tv, side, acc);
+        add_span<L, LAYOUT, CH, ROW * R, (ROW + 1) * R>(bits, tv, side, acc);
+        add_rows<L, LAYOUT, GLOBAL, CH, ROW + 1>(bits, t4, tv, side, acc);
     }
 }
 
 // Accumulate the beta terms of edge e's set dual bits for one endpoint side
 // (tau row loaded as 16-byte vectors; beta1 = tau_signed, beta2 = |tau_signed|),
-// in entry order.
+// in entry order, for CH chains.
 // GLOBAL: the row is in global memory (read-only path); else in shared memory.
+template <int L, int LAYOUT, bool GLOBAL, int CH>
+__device__ __forceinline__ void add_side_chains(const uint32_t (&bits)[CH][Ent<L, LAYOUT>::W],
+                                                const float* __restrict__ tau_e, int side, float (&acc)[CH][L]) {
+    const float4* t4 = reinterpret_cast<const float4*>(tau_e);
+    float tv[Ent<L, LAYOUT>::MP];
+    if (side == 0) add_rows<L, LAYOUT, GLOBAL, CH, 0>(bits, t4, tv, 0, acc);
+    else add_rows<L, LAYOUT, GLOBAL, CH, 0>(bits, t4, tv, 1, acc);
+}
+
 template <int L, int LAYOUT, bool GLOBAL = true>
 __device__ __forceinline__ void add_side(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
                                          int side, float (&acc)[L]) {
-    const float4* t4 = reinterpret_cast<const float4*>(tau_e);
-    float tv[Ent<L, LAYOUT>::MP];
-    if (side == 0) add_rows<L, LAYOUT, GLOBAL, 0>(bits, t4, tv, 0, acc);
-    else add_rows<L, LAYOUT, GLOBAL, 0>(bits, t4, tv, 1, acc);
+    add_side_chains<L, LAYOUT, GLOBAL, 1>(reinterpret_cast<const uint32_t(&)[1][Ent<L, LAYOUT>::W]>(bits), tau_e, side,
+                                          reinterpret_cast<float(&)[1][L]>(acc));
 }
 
 // Compensated (two-sum) flush of a float32 partial sum into a hi/lo pair, used
@@ -761,6 +820,250 @@ __global__ void __launch_bounds__(256, 4) k_primal_warp(SweepArgs a) {
     }
     float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
     xout[g] = (uint8_t)draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl, a.lpv ? a.lpv + g : nullptr);
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// One-batch warp-per-site form with two chains per lane, for tables of one
+// dual word and sites of at most KB incidences: lane l holds chains 2 l and
+// 2 l + 1 of its warp's 64, so one 8-byte load brings both chains' dual words
+// of an incidence, and every tau row, incidence code and unary row serves both.
+// Small tables are bound by this bookkeeping and the label draws, not by the
+// additions: 48^3, 64 chains, L = 2: 73 us (100 us with one chain per lane).
+// Keeps k_primal's order of additions.
+struct PrimalSite {
+    static constexpr int KB = 8;
+    static constexpr int WARPS = 4;                            // 128 threads
+};
+
+template <int L, int LAYOUT, bool POT = false>
+__global__ void __launch_bounds__(128, L <= 6 ? 8 : 6) k_primal_site(SweepArgs a, FastDiv fdG) {
+    using E = Ent<L, LAYOUT>;
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    constexpr int MP = E::MP, KB = PrimalSite::KB;
+    static_assert(E::W == 1 && MP <= 128, "one dual word; a tau row in one 16-byte copy per lane");
+    __shared__ __align__(16) float s_tau[PrimalSite::WARPS][KB][MP];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t groups = fdG.d, un = blockIdx.x * PrimalSite::WARPS + warp;
+    if (un >= (uint32_t)a.N * groups) return;                     // whole warps only
+    const uint32_t v = fdG.div(un), c = (un - v * groups) * 64 + lane * 2;
+    const int64_t p0 = a.inc_ptr[v];
+    const int deg = (int)(a.inc_ptr[v + 1] - p0);
+    const uint32_t code_l = lane < deg ? (uint32_t)__ldg(&a.inc[p0 + lane].x) : 0u;
+    const uint32_t sweep = (uint32_t)a.ctl->sweep;
+    uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
+    const uint32_t* const th0 = a.theta + c;
+    const uint32_t st = (uint32_t)__cvta_generic_to_shared(&s_tau[warp][0][0]) + lane * 16;
+    uint32_t bits[KB][2][1];
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+        if (u < deg) {
+            const uint32_t e = __shfl_sync(FULL, code_l, u) >> 1;
+            const uint2 q = __ldcs(reinterpret_cast<const uint2*>(th0 + (uint64_t)e * (uint32_t)a.C));
+            bits[u][0][0] = q.x;
+            bits[u][1][0] = q.y;
+            if (lane * 4 < MP)
+                cp_async16(st + u * MP * 4, reinterpret_cast<const uint8_t*>(a.tau) + (uint64_t)e * (MP * 4) + lane * 16);
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const float* uf = a.utf + (int64_t)v * L;
+    float ut[L];
+    if constexpr (L % 4 == 0) {
+#pragma unroll
+        for (int x = 0; x < L; x += 4) {
+            const float4 q = __ldg(reinterpret_cast<const float4*>(uf + x));
+            ut[x] = q.x; ut[x + 1] = q.y; ut[x + 2] = q.z; ut[x + 3] = q.w;
+        }
+    } else {
+#pragma unroll
+        for (int x = 0; x < L; ++x) ut[x] = __ldg(uf + x);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
+    float acc[2][L];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int x = 0; x < L; ++x) acc[h][x] = 0.0f;
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+        if (u >= deg) break;
+        const int side = (int)(__shfl_sync(FULL, code_l, u) & 1u);
+        add_side_chains<L, LAYOUT, false, 2>(bits[u], &s_tau[warp][u][0], side, acc);
+    }
+    const int64_t g = (int64_t)v * a.C + c;
+    uint32_t out = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float F[L];
+#pragma unroll
+        for (int x = 0; x < L; ++x) F[x] = ut[x] + acc[h][x];
+        if (POT) {
+            float* pv = a.pot + (int64_t)v * L * a.C + c + h;
+#pragma unroll
+            for (int x = 0; x < L; ++x) pv[(int64_t)x * a.C] = F[x];
+        } else {
+            float* lp = a.logp ? a.logp + ((int64_t)(c + h) * a.N + v) * L : nullptr;
+            out |= (uint32_t)draw_label<L>(F, v, c + h, sweep, a.rk, PH_PRIMAL, lp, a.ctl, a.lpv ? a.lpv + g + h : nullptr) << (8 * h);
+        }
+    }
+    if (!POT) *reinterpret_cast<uint16_t*>(xout + g) = (uint16_t)out;
+}
+
+// Warp-per-site form with its loads in a pipeline, for sites of at most `kb`
+// incidences (every lattice) and 32 CH chains per warp.  A persistent warp
+// walks its (site, chain group) units; the theta rows and tau rows of the next
+// unit's incidences and its unary row are on their way into the other half of
+// the warp's shared-memory buffer (16-byte asynchronous copies) while the
+// current unit is summed, the incidence codes of the unit after that are in a
+// register and the incidence range of the next one too, so no dependent load
+// is waited for.  CH = 2 chains per lane share every tau load and every
+// incidence's bookkeeping.  Keeps k_primal's order of additions.
+// Bound by instruction issue (73 % of the issue slots, 20 warps per SM): 128^3,
+// L = 8, 64 chains: 760 instructions per 32 site updates (968 in the form that
+// loaded a site's incidences when it came to it), 3.54 ms per sweep (4.35 ms).
+template <int L, int LAYOUT, int CH>
+struct PrimalPipe {
+    using E = Ent<L, LAYOUT>;
+    static constexpr int WARPS = 4;                            // 128 threads
+    static constexpr int TH = 32 * CH * E::W * 4;              // bytes of a theta row (32 CH chains)
+    static constexpr int TAU = E::MP * 4;                      // bytes of a tau row
+    static constexpr int UT = 64;                              // bytes kept for the unary row
+    static constexpr int BLOCKS = L <= 8 ? (CH == 2 ? 5 : 8) : 4;   // blocks per SM the registers allow
+    __host__ __device__ static constexpr int stage(int kb) { return kb * (TH + TAU) + UT; }
+    __host__ __device__ static constexpr int smem(int kb) { return WARPS * 2 * stage(kb); }
+};
+
+template <int L, int LAYOUT, int CH, bool POT = false>
+__global__ void __launch_bounds__(128, PrimalPipe<L, LAYOUT, CH>::BLOCKS) k_primal_pipe(SweepArgs a, int kb, FastDiv fdG) {
+    using E = Ent<L, LAYOUT>;
+    using P = PrimalPipe<L, LAYOUT, CH>;
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    constexpr int W = E::W;
+    extern __shared__ __align__(16) uint8_t s_pipe[];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t nw = gridDim.x * P::WARPS;
+    const uint32_t groups = fdG.d, units = (uint32_t)a.N * groups;       // below 2^27: N C < 2^32 (host)
+    const uint32_t first = blockIdx.x * P::WARPS + warp;
+    if (first >= units) return;
+    uint8_t* buf = s_pipe + (size_t)warp * 2 * P::stage(kb);
+    const uint32_t sbuf = (uint32_t)__cvta_generic_to_shared(buf) + lane * 16;
+    const uint32_t sweep = (uint32_t)a.ctl->sweep;
+    uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
+    const uint8_t* const theta_l = reinterpret_cast<const uint8_t*>(a.theta) + lane * 16;
+    const uint8_t* const tau_l = reinterpret_cast<const uint8_t*>(a.tau) + lane * 16;
+    const uint32_t theta_edge = (uint32_t)a.C * (W * 4);
+
+    auto range = [&](uint32_t un, int64_t& p, int& deg) {
+        deg = 0;
+        if (un < units) {
+            const uint32_t v = fdG.div(un);
+            p = a.inc_ptr[v];
+            deg = (int)(a.inc_ptr[v + 1] - p);
+        }
+    };
+    auto codes = [&](int64_t p, int deg) { return lane < deg ? __ldg(&a.inc[p + lane].x) : -1; };
+    // copies of unit `un`, whose incidence codes the lanes hold, into buffer half `half`
+    auto load = [&](uint32_t un, int code, int half) {
+        if (un < units) {
+            const uint32_t v = fdG.div(un), grp = un - v * groups;
+            const int deg = __popc(__ballot_sync(FULL, code >= 0));
+            const uint32_t eu = (uint32_t)code >> 1;
+            const uint8_t* th = theta_l + grp * P::TH;
+            uint32_t dst = sbuf + half * P::stage(kb), dtau = dst + kb * P::TH;
+#pragma unroll 2
+            for (int u = 0; u < deg; ++u, dst += P::TH, dtau += P::TAU) {
+                const uint32_t e = __shfl_sync(FULL, eu, u);
+                const uint8_t* src = th + (uint64_t)e * theta_edge;
+                const uint8_t* tsrc = tau_l + (uint64_t)e * P::TAU;
+#pragma unroll
+                for (int o = 0; o < P::TH; o += 512)
+                    if (o + 512 <= P::TH || o + lane * 16 < P::TH) cp_async16(dst + o, src + o);
+#pragma unroll
+                for (int o = 0; o < P::TAU; o += 512)
+                    if (o + 512 <= P::TAU || o + lane * 16 < P::TAU) cp_async16(dtau + o, tsrc + o);
+            }
+            if (lane < L) cp_async4(sbuf - lane * 12 + half * P::stage(kb) + kb * (P::TH + P::TAU), a.utf + (int64_t)v * L + lane);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    int64_t p = 0;
+    int deg;
+    range(first, p, deg);
+    int code = codes(p, deg);
+    load(first, code, 0);
+    range(first + nw, p, deg);
+    int code1 = codes(p, deg);
+    range(first + 2 * nw, p, deg);
+    int half = 0;
+    for (uint32_t un = first; un < units; un += nw, half ^= 1) {
+        load(un + nw, code1, half ^ 1);
+        const int code2 = codes(p, deg);
+        range(un + 3 * nw, p, deg);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const uint8_t* st = buf + (size_t)half * P::stage(kb);
+        const int n = __popc(__ballot_sync(FULL, code >= 0));
+        float acc[CH][L];
+#pragma unroll
+        for (int h = 0; h < CH; ++h)
+#pragma unroll
+            for (int x = 0; x < L; ++x) acc[h][x] = 0.0f;
+        for (int u = 0; u < n; ++u) {
+            const int side = __shfl_sync(FULL, code, u) & 1;
+            uint32_t bits[CH][W];
+#pragma unroll
+            for (int h = 0; h < CH; ++h) {
+                const uint32_t* th = reinterpret_cast<const uint32_t*>(st + u * P::TH) + (h * 32 + lane) * W;
+                if constexpr (W % 4 == 0) {
+#pragma unroll
+                    for (int w = 0; w < W; w += 4) {
+                        const uint4 q = *reinterpret_cast<const uint4*>(th + w);
+                        bits[h][w] = q.x; bits[h][w + 1] = q.y; bits[h][w + 2] = q.z; bits[h][w + 3] = q.w;
+                    }
+                } else if constexpr (W % 2 == 0) {
+#pragma unroll
+                    for (int w = 0; w < W; w += 2) {
+                        const uint2 q = *reinterpret_cast<const uint2*>(th + w);
+                        bits[h][w] = q.x; bits[h][w + 1] = q.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int w = 0; w < W; ++w) bits[h][w] = th[w];
+                }
+            }
+            add_side_chains<L, LAYOUT, false, CH>(bits, reinterpret_cast<const float*>(st + kb * P::TH + u * P::TAU),
+                                                  side, acc);
+        }
+        const uint32_t v = fdG.div(un), c0 = (un - v * groups) * 32 * CH + lane;
+        const float* ut = reinterpret_cast<const float*>(st + kb * (P::TH + P::TAU));
+#pragma unroll
+        for (int h = 0; h < CH; ++h) {
+            const uint32_t c = c0 + 32 * h;
+            float F[L];
+#pragma unroll
+            for (int x = 0; x < L; ++x) F[x] = ut[x] + acc[h][x];
+            if (POT) {
+                float* pv = a.pot + (int64_t)v * L * a.C + c;
+#pragma unroll
+                for (int x = 0; x < L; ++x) pv[(int64_t)x * a.C] = F[x];
+            } else {
+                const int64_t g = (int64_t)v * a.C + c;
+                float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
+                xout[g] = (uint8_t)draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl, a.lpv ? a.lpv + g : nullptr);
+            }
+        }
+        __syncwarp();                                                    // this half is free for the unit after the next
+        code = code1;
+        code1 = code2;
+    }
 }
 
 // CTA-per-site schedule of the plain primal step for high-degree sites: a CTA
@@ -1240,17 +1543,62 @@ cudaError_t run_dual(const SweepArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// The pipelined warp form where its buffers leave at least two blocks per SM; false if not.
+template <int L, int LAYOUT, int CH, bool POT>
+bool try_primal_pipe(const SweepArgs& a, cudaStream_t s, cudaError_t& e) {
+    using P = PrimalPipe<L, LAYOUT, CH>;
+    if (a.C % (32 * CH) || a.max_deg >= 32) return false;
+    const int kb = a.max_deg > 0 ? a.max_deg : 1, smem = P::smem(kb);
+    if (smem > 100 * 1024) return false;
+    if (smem > 48 * 1024) {
+        e = cudaFuncSetAttribute(k_primal_pipe<L, LAYOUT, CH, POT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return true;
+    }
+    const int64_t blocks = ((int64_t)a.N * (a.C / (32 * CH)) + P::WARPS - 1) / P::WARPS;
+    const int64_t resident = 152 * std::min<int64_t>(P::BLOCKS, 227 * 1024 / (smem + 1024));
+    k_primal_pipe<L, LAYOUT, CH, POT><<<(unsigned)std::min(blocks, resident), 32 * P::WARPS, smem, s>>>(
+        a, kb, FastDiv::make((uint32_t)(a.C / (32 * CH))));
+    e = cudaGetLastError();
+    return true;
+}
+
+// Chains a multiple of 32: the warp form by table width, degree and chains.
+// us per launch on a 48^3 lattice (degree 6), measured one against the other:
+//   one dual word, L <= 8, 64 chains: two chains per lane (k_primal_site) 73 / 98 / 114 / 127 for
+//     L = 2 / 4 / 5 / 6 against 100 / 118 / 134 / 149 with one chain per lane (k_primal_warp);
+//     with 16 labels on the diagonal 194 against 170, so one chain per lane there
+//   PIVOT, L = 7 ... 12, 64 chains: pipelined, two chains per lane 165 / 191 / 252 / 284 / 366 / 409 (L = 8: 191)
+//     against 189 / 215 / 268 / 310 / 506 / 546
+//   PIVOT, L = 11 ... 14, 32 chains: pipelined, one chain per lane 199 / 221 / - / 329 against
+//     260 / 282 / - / 375; for L <= 10 it is slower (L = 8: 135 against 115), L = 16 even (527 and 525)
+template <int L, int LAYOUT, bool POT>
+cudaError_t run_primal_warps(const SweepArgs& a, cudaStream_t s) {
+    const int64_t n = (int64_t)a.N * a.C;
+    cudaError_t e = cudaSuccess;
+    if constexpr (Ent<L, LAYOUT>::W == 1 && L <= 8) {
+        if (a.C % 64 == 0 && a.max_deg <= PrimalSite::KB) {
+            k_primal_site<L, LAYOUT, POT><<<blocks_for(n, 64 * PrimalSite::WARPS), 32 * PrimalSite::WARPS, 0, s>>>(
+                a, FastDiv::make((uint32_t)(a.C / 64)));
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (LAYOUT == MRF_LAYOUT_PIVOT && L >= 7 && L <= 12)
+        if (try_primal_pipe<L, LAYOUT, 2, POT>(a, s, e)) return e;
+    if constexpr (LAYOUT == MRF_LAYOUT_PIVOT && L >= 11 && L <= 14)
+        if (try_primal_pipe<L, LAYOUT, 1, POT>(a, s, e)) return e;
+    if (a.max_deg <= PrimalWarp<L, LAYOUT>::KB)
+        k_primal_warp<L, LAYOUT, POT, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
+    else
+        k_primal_warp<L, LAYOUT, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
 template <int L, int LAYOUT, bool FUSED>
 cudaError_t run_primal(const SweepArgs& a, cudaStream_t s) {
     const int64_t n = (int64_t)a.N * a.C;
     if (n <= 0) return cudaSuccess;
-    if (!FUSED && a.C % 32 == 0) {
-        if (a.max_deg <= PrimalWarp<L, LAYOUT>::KB)
-            k_primal_warp<L, LAYOUT, false, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
-        else
-            k_primal_warp<L, LAYOUT><<<blocks_for(n, 256), 256, 0, s>>>(a);
-    } else
-        k_primal<L, LAYOUT, FUSED><<<blocks_for(n, 256), 256, 0, s>>>(a);
+    if (!FUSED && a.C % 32 == 0) return run_primal_warps<L, LAYOUT, false>(a, s);
+    k_primal<L, LAYOUT, FUSED><<<blocks_for(n, 256), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1258,13 +1606,8 @@ template <int L, int LAYOUT>
 cudaError_t run_potential(const SweepArgs& a, cudaStream_t s) {
     const int64_t n = (int64_t)a.N * a.C;
     if (n <= 0) return cudaSuccess;
-    if (a.C % 32 == 0) {
-        if (a.max_deg <= PrimalWarp<L, LAYOUT>::KB)
-            k_primal_warp<L, LAYOUT, true, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
-        else
-            k_primal_warp<L, LAYOUT, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
-    } else
-        k_primal<L, LAYOUT, false, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
+    if (a.C % 32 == 0) return run_primal_warps<L, LAYOUT, true>(a, s);
+    k_primal<L, LAYOUT, false, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,72 @@
+"""Forms of the sweep kernels that are chosen by size, against the oracle: one
+plain sweep's labels without the log-probability record (so the label draw
+takes its short form first), tolerance the parity protocol's 1e-6 around a
+decision boundary."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from oracle import decompose as dc, sampler
+from paper_1611_06684_gb300 import workloads as wl
+from paper_1611_06684_gb300 import mrf as M
+from tests.gpu_helpers import make_handle, compare_sweep
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1611_06684_gb300 import build
+    build.build()
+    torch.cuda.set_device(0)
+
+
+def _check(model, C, seed, t=3, **kw):
+    h = make_handle(model, C, seed, use_graphs=False, schedule=kw.pop("schedule", 1), **kw)
+    x0 = h.get_labels()
+    h.set_sweep_index(t)
+    h.sweep(1, M.MODE_PLAIN)
+    dec = dc.decompose(model)
+    ref = sampler.sweep(dec, x0.astype(np.int64), t, seed)
+    W = (dec.ell.shape[1] + 31) // 32
+    theta = M.unpack_theta(h.debug_theta(), dec.ell.shape[1]) if model.n_edges else None
+    stats = compare_sweep(dec, ref, h.get_labels(), theta_gpu=theta)
+    seen, expect = h.boundary_draws(), stats["site_boundary"]
+    h.close()
+    # the device's count uses its float32 CDF: a draw at the edge of the 1e-6 band may differ
+    assert abs(int(seen) - expect) <= 3 + expect, (seen, expect)
+
+
+def _wide_fields(L, seed):
+    """Unaries from 0 to 3e4 in magnitude, exact ties among them."""
+    m = wl.potts_grid3d(5, 4, 3, L=L, seed=seed)
+    rng = np.random.default_rng(seed)
+    m.unary *= np.float32(10.0) ** rng.integers(-1, 5, (m.n_vars, 1)).astype(np.float32)
+    m.unary[::3] = np.round(m.unary[::3, :1])
+    return m
+
+
+@pytest.mark.parametrize("L,C,shape", [(2, 64, (7, 5, 3)), (3, 128, (9, 1, 1)), (4, 64, (5, 5, 1)), (6, 64, (6, 3, 2)),
+                                       (7, 64, (5, 4, 3)), (8, 192, (4, 3, 3)), (10, 64, (5, 3, 2)), (12, 64, (4, 3, 2)),
+                                       (11, 32, (4, 3, 3)), (12, 96, (3, 3, 3)), (14, 32, (4, 3, 2)), (8, 32, (5, 4, 3)),
+                                       (16, 64, (3, 3, 2)), (5, 24, (5, 4, 3))])
+def test_lattice_forms_match_the_oracle(L, C, shape):
+    _check(wl.potts_grid3d(*shape, L=L, seed=40 + L), C, 1000 + L)
+
+
+@pytest.mark.parametrize("L,C", [(4, 64), (8, 64), (8, 32), (16, 64)])
+def test_diagonal_tables_match_the_oracle(L, C):
+    _check(wl.ferro_potts_grid3d(5, 4, 3, L=L, seed=50 + L), C, 2000 + L)
+
+
+@pytest.mark.parametrize("L,C,E", [(8, 64, 150), (5, 64, 400), (12, 32, 120)])
+def test_sites_of_uneven_degree_match_the_oracle(L, C, E):
+    # isolated sites and degrees on both sides of the one-batch and pipelined forms' limits
+    _check(wl.tiny_random(60, L, E, w_std=0.4, seed=60 + L), C, 3000 + L)
+
+
+@pytest.mark.parametrize("L,C", [(2, 64), (8, 64), (8, 5), (16, 32)])
+def test_label_draw_of_wide_fields_matches_the_oracle(L, C):
+    _check(_wide_fields(L, 70 + L), C, 4000 + L)
