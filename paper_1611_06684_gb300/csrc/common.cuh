@@ -40,8 +40,11 @@ struct Ctl {
     unsigned long long sweep;          // index t of the sweep being run / next
     unsigned long long count_from;     // sweeps with t >= count_from are counted
     unsigned long long boundary;       // draws within 1e-6 of a decision boundary
-    unsigned long long splash_offset;  // packed (ox | oy << 8 | oz << 16) of the last blocked sweep
+    uint32_t splash_offset;            // packed (ox | oy << 8 | oz << 16) of the last blocked sweep
+    uint32_t done;                     // clusters of a small-model launch that have finished (0 between launches)
 };
+
+static_assert(sizeof(Ctl) == 32, "part of the checkpoint format");
 
 // Division by a fixed 32-bit divisor d via a multiply (Granlund & Montgomery,
 // "Division by invariant integers using multiplication", 1994):
@@ -233,7 +236,6 @@ cudaError_t launch_accumulate(const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_philox_rate(uint64_t threads, int calls, uint32_t* sink, cudaStream_t s);
 cudaError_t launch_log_v(const SweepArgs& a, const double* ut, double* out, cudaStream_t s);
 cudaError_t launch_em(const SweepArgs& a, int layout, const uint8_t* xin, uint8_t* xout, cudaStream_t s);
-int64_t sweep_small_smem(const SweepArgs& a);
 cudaError_t launch_sweep_small(const SweepArgs& a, int layout, int n_sweeps, cudaStream_t s);
 cudaError_t launch_mf(const SweepArgs& a, int layout, const float* qin, float* qout, cudaStream_t s);
 cudaError_t launch_marg_layout(const float* in, float* out, int N, int L, int C, bool to_abi, cudaStream_t s);

@@ -757,14 +757,15 @@ static mrf_status tune_schedule(mrf_t* h) {
 
 static bool use_mlp_tc(const mrf_t* h) { return h->opt.mlp_path == 0 && mlp_tc_supported(h->la); }
 
-// Models small enough for k_sweep_small: at most 2^16 (site, chain) and
-// (edge, chain) items, theta of all items within 200 KB of shared memory.
-// Small models run several plain sweeps in one single-CTA launch (k_sweep_small,
-// the additions of k_primal); handles on the edge-partial form keep it for
-// every sweep, so that a chain does not depend on the sweeps per call.
+// Small models (at most 2^16 (site, chain) and (edge, chain) items) run several
+// plain sweeps in one launch (k_sweep_resident, k_sweep_small: the additions of
+// k_primal).  The limit is where a launch per half-step wins again: a 12^3
+// lattice, L = 8, 32 chains (165,888 edge items): 208 us per 10 sweeps in separate
+// launches, 382 us in one.  Handles on the edge-partial form keep it for every
+// sweep, so that a chain does not depend on the sweeps per call.
 static bool small_model(const mrf_t* h) {
     const int64_t nv = (int64_t)h->N * h->C, ne = h->E_slots * h->C;
-    return nv <= 65536 && ne <= 65536 && ne * h->W * 4 <= 200 * 1024 && !use_partial(h);
+    return nv <= 65536 && ne <= 65536 && !use_partial(h);
 }
 
 static SwArgs make_sw_args(const mrf_t* h) {

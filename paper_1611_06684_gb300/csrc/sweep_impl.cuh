@@ -137,22 +137,41 @@ __device__ __forceinline__ void pivot_masks64(int xs, int xt, uint64_t& Y, uint6
 // Returns lt in bits, the ties le & ~lt (probability 1/256 per entry) in ties
 // and the level-2 mask in lev2; a tie is decided by the low 16 bits of its
 // uniform against the exact threshold of its level (resolve_tie).
+// The Philox calls of the table's first two groups (draw_dual_words) do not
+// depend on the labels and come as an argument.
+// GLOBAL: the plane table is in global memory (read-only path); else in shared memory.
 template <int L, int LAYOUT>
+struct DualWords {
+    static constexpr int GA = Ent<L, LAYOUT>::W < 2 ? Ent<L, LAYOUT>::W : 2;   // groups drawn together
+    static constexpr int N = Ent<L, LAYOUT>::M <= 16 ? 1 : 2 * GA;
+};
+
+template <int L, int LAYOUT>
+__device__ __forceinline__ void draw_dual_words(uint32_t e, uint32_t c, uint32_t sweep, const RoundKeys& key,
+                                                uint4 (&R)[DualWords<L, LAYOUT>::N]) {
+    // four calls of two groups share their first rounds and are in flight together
+    if constexpr (DualWords<L, LAYOUT>::N == 1) R[0] = draw_rk(e, sweep, c, PH_DUAL, 0u, key);
+    else draw_rk_subs<DualWords<L, LAYOUT>::N>(e, sweep, c, PH_DUAL, key, R);
+}
+
+template <int L, int LAYOUT, bool GLOBAL = true>
 __device__ __forceinline__ void dual_prefix_bits(uint32_t e, uint32_t c, int xs, int xt,
                                                  const uint32_t* __restrict__ tpl_e, uint32_t sweep,
                                                  const RoundKeys& key, uint32_t (&bits)[Ent<L, LAYOUT>::W],
                                                  uint32_t (&ties)[Ent<L, LAYOUT>::W],
-                                                 uint32_t (&lev2)[Ent<L, LAYOUT>::W]) {
+                                                 uint32_t (&lev2)[Ent<L, LAYOUT>::W],
+                                                 const uint4 (&RA)[DualWords<L, LAYOUT>::N]) {
     using E = Ent<L, LAYOUT>;
     const uint4* tp = reinterpret_cast<const uint4*>(tpl_e);
+    auto table = [](const uint4* q) { return GLOBAL ? __ldg(q) : *q; };
     if constexpr (E::M <= 16) {
         // one Philox call: word p = plane p (bits 0..15) and plane p + 4 (bits
         // 16..31); the low halves compare the prefix's high nibble, the high
         // halves its low nibble, combined at the end
-        const uint4 r4 = draw_rk(e, sweep, c, PH_DUAL, 0u, key);
+        const uint4 r4 = RA[0];
         const uint32_t R[4] = {r4.x, r4.y, r4.z, r4.w};
-        const uint4 qa = __ldg(tp), qb = __ldg(tp + 1);
-        const uint32_t sa = __ldg(tpl_e + 8);
+        const uint4 qa = table(tp), qb = table(tp + 1);
+        const uint32_t sa = GLOBAL ? __ldg(tpl_e + 8) : tpl_e[8];
         const uint32_t AB[4] = {qa.x, qa.y, qa.z, qa.w}, B[4] = {qb.x, qb.y, qb.z, qb.w};
         const uint32_t Y = row_mask<L, LAYOUT>(xs, 0), Z = col_mask<L, LAYOUT>(xt, 0);
         const uint32_t X = (sa & 0xFFFFu) ^ Y, act = sa >> 16;
@@ -174,10 +193,7 @@ __device__ __forceinline__ void dual_prefix_bits(uint32_t e, uint32_t c, int xs,
     constexpr bool M64 = LAYOUT == MRF_LAYOUT_PIVOT && E::M <= 64;
     uint64_t Y64 = 0, Z64 = 0;
     if constexpr (M64) pivot_masks64<L>(xs, xt, Y64, Z64);
-    // the first two groups' four Philox calls share their first rounds and are in flight together
-    constexpr int GA = E::W < 2 ? E::W : 2;
-    uint4 RA[2 * GA];
-    draw_rk_subs<2 * GA>(e, sweep, c, PH_DUAL, key, RA);
+    constexpr int GA = DualWords<L, LAYOUT>::GA;
 #pragma unroll
     for (int g = 0; g < E::W; ++g) {
         uint4 r0, r1;
@@ -190,7 +206,7 @@ __device__ __forceinline__ void dual_prefix_bits(uint32_t e, uint32_t c, int xs,
         }
         const uint32_t Rg[8] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w};
         const uint4* tg = tp + 5 * g;
-        const uint4 sq = __ldg(tg + 4);                    // {S, Act}
+        const uint4 sq = table(tg + 4);                    // {S, Act}
         uint32_t Y, Z;
         if constexpr (M64) {
             Y = (uint32_t)(Y64 >> (32 * g));
@@ -204,7 +220,7 @@ __device__ __forceinline__ void dual_prefix_bits(uint32_t e, uint32_t c, int xs,
         uint32_t lt = 0u, le = 0xFFFFFFFFu;
 #pragma unroll
         for (int h = 3; h >= 0; --h) {
-            const uint4 q = __ldg(tg + h);                 // {AB_2h, B_2h, AB_2h+1, B_2h+1}
+            const uint4 q = table(tg + h);                 // {AB_2h, B_2h, AB_2h+1, B_2h+1}
             uint32_t t = q.w ^ (q.z & L0), r = Rg[2 * h + 1];
             lt = (~r & t) | (~(r ^ t) & lt);
             le = (~r & t) | (~(r ^ t) & le);
@@ -227,14 +243,16 @@ __device__ __forceinline__ bool resolve_tie(uint32_t e, uint32_t c, bool lev2, i
     return rem && dual_low16(e, sweep, c, k, key) < rem;
 }
 
-// Dual bits with the ties decided by the thread itself, one after another.
-template <int L, int LAYOUT>
+// Dual bits with the ties decided by the thread itself, one after another
+// (thr_e in global memory, or both tables in shared memory).
+template <int L, int LAYOUT, bool GLOBAL = true>
 __device__ __forceinline__ void dual_bits(uint32_t e, uint32_t c, int xs, int xt, const uint32_t* __restrict__ tpl_e,
                                           const uint32_t* __restrict__ thr_e, uint32_t sweep, const RoundKeys& key,
-                                          uint32_t (&bits)[Ent<L, LAYOUT>::W]) {
+                                          uint32_t (&bits)[Ent<L, LAYOUT>::W],
+                                          const uint4 (&R)[DualWords<L, LAYOUT>::N]) {
     using E = Ent<L, LAYOUT>;
     uint32_t ties[E::W], lev2[E::W];
-    dual_prefix_bits<L, LAYOUT>(e, c, xs, xt, tpl_e, sweep, key, bits, ties, lev2);
+    dual_prefix_bits<L, LAYOUT, GLOBAL>(e, c, xs, xt, tpl_e, sweep, key, bits, ties, lev2, R);
 #pragma unroll 1
     for (int g = 0; g < E::W; ++g) {
         uint32_t tg = ties[g];
@@ -242,9 +260,18 @@ __device__ __forceinline__ void dual_bits(uint32_t e, uint32_t c, int xs, int xt
             const int b = __ffs(tg) - 1;
             tg &= tg - 1u;
             const int k = 32 * g + b;
-            if (resolve_tie(e, c, (lev2[g] >> b) & 1u, k, __ldg(thr_e + k), sweep, key)) bits[g] |= 1u << b;
+            if (resolve_tie(e, c, (lev2[g] >> b) & 1u, k, GLOBAL ? __ldg(thr_e + k) : thr_e[k], sweep, key)) bits[g] |= 1u << b;
         }
     }
+}
+
+template <int L, int LAYOUT>
+__device__ __forceinline__ void dual_bits(uint32_t e, uint32_t c, int xs, int xt, const uint32_t* __restrict__ tpl_e,
+                                          const uint32_t* __restrict__ thr_e, uint32_t sweep, const RoundKeys& key,
+                                          uint32_t (&bits)[Ent<L, LAYOUT>::W]) {
+    uint4 R[DualWords<L, LAYOUT>::N];
+    draw_dual_words<L, LAYOUT>(e, c, sweep, key, R);
+    dual_bits<L, LAYOUT, true>(e, c, xs, xt, tpl_e, thr_e, sweep, key, bits, R);
 }
 
 // ---------------------------------------------------------------------------- label draw
@@ -293,15 +320,12 @@ __device__ __forceinline__ int draw_label_fast(const float (&F)[L], float u) {
     return closest >= s * 0x1p-16f ? lab : -1;
 }
 
-// Draw x_v from exp(F)/Z by the inverse CDF with the 23-bit uniform u of
-// Philox phase `phase` (u is exact in float32); optionally record log p.
-// Counts draws within 1e-6 of a CDF boundary.
-// lp_drawn (optional) receives log p of the drawn label.
+// Draw x_v from exp(F)/Z by the inverse CDF with the 23-bit uniform u (exact in
+// float32); optionally record log p.  Counts draws within 1e-6 of a CDF
+// boundary.  lp_drawn (optional) receives log p of the drawn label.
 template <int L>
-__device__ __forceinline__ int draw_label(const float (&F)[L], uint32_t v, uint32_t c, uint32_t sweep,
-                                          const RoundKeys& key, uint32_t phase, float* __restrict__ logp_out, Ctl* ctl,
-                                          float* __restrict__ lp_drawn = nullptr) {
-    const float u = uniform23(draw_rk(v, sweep, c, phase, 0, key).x);
+__device__ __forceinline__ int draw_label_at(const float (&F)[L], float u, float* __restrict__ logp_out, Ctl* ctl,
+                                             float* __restrict__ lp_drawn = nullptr) {
     if (!logp_out && !lp_drawn) {
         const int lab = draw_label_fast<L>(F, u);
         if (lab >= 0) return lab;
@@ -342,6 +366,14 @@ __device__ __forceinline__ int draw_label(const float (&F)[L], uint32_t v, uint3
         *lp_drawn = (fp - mx) - logf(s);
     }
     return pick;
+}
+
+// The same with the uniform of Philox phase `phase` for site v, chain c.
+template <int L>
+__device__ __forceinline__ int draw_label(const float (&F)[L], uint32_t v, uint32_t c, uint32_t sweep,
+                                          const RoundKeys& key, uint32_t phase, float* __restrict__ logp_out, Ctl* ctl,
+                                          float* __restrict__ lp_drawn = nullptr) {
+    return draw_label_at<L>(F, uniform23(draw_rk(v, sweep, c, phase, 0, key).x), logp_out, ctl, lp_drawn);
 }
 
 // ---------------------------------------------------------------------------- kernels
@@ -392,7 +424,9 @@ __global__ void __launch_bounds__(256, FEW ? 2 : 4) k_dual(SweepArgs a) {
         if (s >= 0 && !(a.splash && is_tree_edge(a, e)) && !(a.skip && a.skip[e])) {
             const int t = a.dst[e];
             const int xs = xin[(int64_t)s * a.C + c], xt = xin[(int64_t)t * a.C + c];
-            dual_prefix_bits<L, LAYOUT>(e, c, xs, xt, a.tpl + (int64_t)e * E::PW, sweep, a.rk, bits, ties, lev2);
+            uint4 R[DualWords<L, LAYOUT>::N];
+            draw_dual_words<L, LAYOUT>(e, c, sweep, a.rk, R);
+            dual_prefix_bits<L, LAYOUT>(e, c, xs, xt, a.tpl + (int64_t)e * E::PW, sweep, a.rk, bits, ties, lev2, R);
         } else {
 #pragma unroll
             for (int w = 0; w < W; ++w) { bits[w] = 0u; ties[w] = 0u; lev2[w] = 0u; }
@@ -1281,56 +1315,102 @@ cudaError_t run_sweep_partial(const SweepArgs& a, int step, cudaStream_t s) {
 
 // ---------------------------------------------------------------------------- small models
 
-// n_sweeps whole plain sweeps of a small model in one CTA (sizes where launch
-// latency, not work, sets the time): dual half-step into shared memory,
-// primal half-step, marginal counts and the sweep advance, separated by CTA
-// barriers only.  The draws and the order of every addition are those of
-// k_dual / k_primal, so the chain is the same bit for bit.
+// Barrier of a thread-block cluster: what its threads wrote before is seen by
+// its threads after (loads that may have been cached go to L2).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+__device__ __forceinline__ void cluster_barrier() { cluster_arrive(); cluster_wait(); }
+
+// Dual words of one (edge, chain) and one incidence side, from L2.
+template <int W>
+__device__ __forceinline__ void load_words_cg(const uint32_t* th, uint32_t (&bits)[W]) {
+    if constexpr (W % 2 == 0) {
+#pragma unroll
+        for (int w = 0; w < W; w += 2) {
+            const uint2 q = __ldcg(reinterpret_cast<const uint2*>(th + w));
+            bits[w] = q.x;
+            bits[w + 1] = q.y;
+        }
+    } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) bits[w] = __ldcg(th + w);
+    }
+}
+
+// n_sweeps whole plain sweeps of a small model in one launch (sizes where
+// launches and latency, not work, set the time).  Chains are independent, so
+// a cluster of CTAs takes nc chains and no cluster waits for another; within
+// it the items of a half-step are spread over all its threads, labels and
+// dual bits go through L2, and the half-steps are separated by cluster
+// barriers only.  Counts are reductions to memory from the label draw.  The
+// draws and the order of every addition are those of k_dual / k_primal, so
+// the chain is the same bit for bit.  The sweep index is read from device
+// memory by every thread and advanced by the last cluster to finish.
+// Bound by latency (two barriers and their dependent L2 round trips).  50 x 50
+// Ising grid, 10 chains, 10 sweeps: 990 us in one CTA with all chains, 62 us here.
 template <int L, int LAYOUT>
-__global__ void __launch_bounds__(1024) k_sweep_small(SweepArgs a, int n_sweeps) {
+__global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, FastDiv fdn) {
     using E = Ent<L, LAYOUT>;
-    extern __shared__ uint32_t s_theta[];                          // [E][C][W]
-    const int64_t ne = a.E * a.C, nv = (int64_t)a.N * a.C;
+    constexpr int W = E::W;
+    uint32_t rank, size;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(size));
+    const uint32_t nc = fdn.d, cluster = blockIdx.x / size;
+    const uint32_t c0 = cluster * nc;
+    const uint32_t tid = rank * blockDim.x + threadIdx.x, T = size * blockDim.x;
+    const uint32_t ne = (uint32_t)a.E * nc, nv = (uint32_t)a.N * nc, C = (uint32_t)a.C;
     uint32_t sweep = (uint32_t)a.ctl->sweep;
     const unsigned long long count_from = a.ctl->count_from;
     for (int it = 0; it < n_sweeps; ++it, ++sweep) {
         const uint8_t* xin = a.x + (size_t)(sweep & 1) * a.N * a.C;
         uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
-        for (int64_t g = threadIdx.x; g < ne; g += blockDim.x) {
-            const uint32_t e = a.fdC.div((uint32_t)g), c = (uint32_t)g - e * (uint32_t)a.C;
-            uint32_t bits[E::W];
+        for (uint32_t i = tid; i < ne; i += T) {
+            const uint32_t e = fdn.div(i), c = c0 + (i - e * nc);
+            if (c >= C) continue;
+            uint32_t bits[W];
             const int s = a.src[e];
             if (s >= 0) {
                 const int t = a.dst[e];
-                dual_bits<L, LAYOUT>(e, c, xin[(int64_t)s * a.C + c], xin[(int64_t)t * a.C + c],
+                dual_bits<L, LAYOUT>(e, c, __ldcg(xin + (int64_t)s * C + c), __ldcg(xin + (int64_t)t * C + c),
                                      a.tpl + (int64_t)e * E::PW, a.thr + (int64_t)e * E::M, sweep, a.rk, bits);
             } else {
 #pragma unroll
-                for (int w = 0; w < E::W; ++w) bits[w] = 0;
+                for (int w = 0; w < W; ++w) bits[w] = 0;
             }
+            uint32_t* out = a.theta + ((int64_t)e * C + c) * W;
 #pragma unroll
-            for (int w = 0; w < E::W; ++w) s_theta[g * E::W + w] = bits[w];
+            for (int w = 0; w < W; ++w) __stcg(out + w, bits[w]);
         }
-        __syncthreads();
-        for (int64_t g = threadIdx.x; g < nv; g += blockDim.x) {
-            const uint32_t v = a.fdC.div((uint32_t)g), c = (uint32_t)g - v * (uint32_t)a.C;
+        if (size > 1) cluster_barrier();
+        else __syncthreads();
+        for (uint32_t i = tid; i < nv; i += T) {
+            const uint32_t v = fdn.div(i), c = c0 + (i - v * nc);
+            if (c >= C) continue;
             float acc[L], hi[L], lo[L];
 #pragma unroll
             for (int x = 0; x < L; ++x) { acc[x] = 0.0f; hi[x] = 0.0f; lo[x] = 0.0f; }
             int chunk = 0;
             bool flushed = false;
-            for (int64_t p = a.inc_ptr[v]; p < a.inc_ptr[v + 1]; ++p) {
-                const int2 ic = __ldg(&a.inc[p]);
-                const int64_t e = ic.x >> 1;
-                uint32_t bits[E::W];
+            const int64_t p0 = a.inc_ptr[v], p1 = a.inc_ptr[v + 1];
+            constexpr int B = W <= 2 ? 4 : 2;              // incidences whose dual words are loaded together
+            for (int64_t base = p0; base < p1; base += B) {
+                int code[B];
+                uint32_t bits[B][W];
 #pragma unroll
-                for (int w = 0; w < E::W; ++w) bits[w] = s_theta[(e * a.C + c) * E::W + w];
-                add_side<L, LAYOUT>(bits, a.tau + e * E::MP, ic.x & 1, acc);
-                if (++chunk == 32) {
+                for (int u = 0; u < B; ++u) code[u] = base + u < p1 ? __ldg(&a.inc[base + u].x) : -1;
 #pragma unroll
-                    for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], acc[x]); acc[x] = 0.0f; }
-                    chunk = 0;
-                    flushed = true;
+                for (int u = 0; u < B; ++u)
+                    if (code[u] >= 0) load_words_cg<W>(a.theta + ((int64_t)(code[u] >> 1) * C + c) * W, bits[u]);
+#pragma unroll
+                for (int u = 0; u < B; ++u) {
+                    if (code[u] < 0) continue;
+                    add_side<L, LAYOUT>(bits[u], a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
+                    if (++chunk == 32) {
+#pragma unroll
+                        for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], acc[x]); acc[x] = 0.0f; }
+                        chunk = 0;
+                        flushed = true;
+                    }
                 }
             }
             float F[L];
@@ -1343,26 +1423,202 @@ __global__ void __launch_bounds__(1024) k_sweep_small(SweepArgs a, int n_sweeps)
                 for (int x = 0; x < L; ++x) F[x] = __ldg(uf + x) + acc[x];
             }
             float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
-            xout[g] = (uint8_t)draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl);
+            const int lab = draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl);
+            __stcg(xout + (int64_t)v * C + c, (uint8_t)lab);
+            if (sweep >= count_from) atomicAdd(a.counts + (int64_t)v * L + lab, 1u);
         }
-        __syncthreads();
-        if (sweep >= count_from) {
-            for (int64_t v = threadIdx.x; v < a.N; v += blockDim.x) {
-                uint32_t tot[L];
+        if (size > 1) cluster_barrier();
+        else __syncthreads();
+    }
+    // after the last barrier every thread of the cluster has read the index
+    if (rank == 0 && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&a.ctl->done, 1u) + 1u == gridDim.x / size) {
+            a.ctl->done = 0u;
+            a.ctl->sweep = sweep;
+        }
+    }
+}
+
+// The same for models small enough that every thread of a cluster owns at
+// most one (edge, chain) and one (site, chain) item: everything the sweeps read
+// stays on the SMs.  Every CTA keeps all labels of the cluster's chains, and
+// the dual words of its own sites' incidences at their (edge, chain) place; a
+// label is stored into every CTA's copy and a dual word into the copies of the
+// two endpoints' owners (distributed shared memory), so that all loads of a
+// half-step are local and its only wait is the barrier.  The plane and
+// threshold words of a thread's edge and the weights of its site's first
+// incidences are staged in shared memory, the edge's endpoints and those
+// incidences' codes in registers (a barrier's acquire drops the L1 lines, so a
+// table word read from memory would be an L2 round trip in every sweep), and
+// the random words of the next half-step are drawn between a barrier's arrival
+// and its wait.  Bound by the latency of the two barriers and of the dual ->
+// label -> dual chain: 32 x 32 Ising grid, one chain: 1.9 us per sweep (4.9 us in
+// one CTA; 4.6 us in k_sweep_small); 50 x 50, 10 chains: 3.4 us (99 us).
+template <int L, int LAYOUT>
+struct SmallResident {
+    using E = Ent<L, LAYOUT>;
+    // words of a thread's table row: plane words and thresholds of its edge, the weights of its site's
+    // first KT incidences (tables of at most 16 entries); an odd number of 16-byte units, so that rows
+    // fall on different banks
+    static constexpr int KT = E::M <= 16 ? 4 : 0;
+    static constexpr int TAU = (E::PW + E::M + 3) / 4 * 4;
+    static constexpr int ROW = ((TAU + KT * E::MP) / 4 | 1) * 4;
+    static int64_t labels(int64_t items) { return (items + 15) / 16 * 16; }
+    static int64_t smem(int64_t site_items, int64_t edge_items, int threads) {
+        return 2 * labels(site_items) + (edge_items * E::W + 3) / 4 * 16 + (int64_t)threads * ROW * 4;
+    }
+};
+
+__device__ __forceinline__ uint32_t cluster_address(uint32_t shared_address, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0,%1,%2;" : "=r"(r) : "r"(shared_address), "r"(rank));
+    return r;
+}
+
+template <int L, int LAYOUT>
+__global__ void __launch_bounds__(640) k_sweep_resident(SweepArgs a, int n_sweeps, FastDiv fdn) {
+    using E = Ent<L, LAYOUT>;
+    using S = SmallResident<L, LAYOUT>;
+    constexpr int W = E::W, KI = 4;                        // incidences kept in registers
+    extern __shared__ __align__(16) uint8_t s_small[];
+    uint32_t rank, size;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(size));
+    const uint32_t nc = fdn.d, c0 = blockIdx.x / size * nc, C = (uint32_t)a.C;
+    const uint32_t i = rank * blockDim.x + threadIdx.x;    // this thread's edge item and site item
+    const uint32_t ne = (uint32_t)a.E * nc, nv = (uint32_t)a.N * nc;
+    const uint32_t lab_bytes = (nv + 15u) / 16u * 16u;
+    uint8_t* s_lab = s_small;                              // [2][N][nc]
+    uint32_t* s_th = reinterpret_cast<uint32_t*>(s_small + 2 * lab_bytes);     // [E][nc][W]
+    uint32_t* s_row = s_th + (ne * W + 3u) / 4u * 4u + threadIdx.x * S::ROW;   // this thread's table row
+    const uint32_t lab_addr = (uint32_t)__cvta_generic_to_shared(s_lab);
+    const uint32_t th_addr = (uint32_t)__cvta_generic_to_shared(s_th);
+    uint32_t sweep = (uint32_t)a.ctl->sweep;
+    const unsigned long long count_from = a.ctl->count_from;
+    const uint8_t* x0 = a.x + (size_t)(sweep & 1) * a.N * a.C;
+    for (uint32_t j = threadIdx.x; j < nv; j += blockDim.x) {
+        const uint32_t v = fdn.div(j), c = c0 + (j - v * nc);
+        s_lab[(sweep & 1) * lab_bytes + j] = c < C ? x0[(int64_t)v * C + c] : 0;
+    }
+    // edge item
+    const uint32_t e = fdn.div(i), ec = c0 + (i - e * nc);
+    const bool has_edge = i < ne && ec < C && a.src[i < ne ? e : 0] >= 0;
+    uint32_t ls = 0, lt = 0, th_s = 0, th_t = 0;           // label places of the endpoints, dual words in their owners' copies
+    if (has_edge) {
+        ls = (uint32_t)a.src[e] * nc + (ec - c0);
+        lt = (uint32_t)a.dst[e] * nc + (ec - c0);
+        th_s = cluster_address(th_addr + i * W * 4, ls / blockDim.x);
+        th_t = cluster_address(th_addr + i * W * 4, lt / blockDim.x);
+        for (int k = 0; k < E::PW; ++k) s_row[k] = __ldg(a.tpl + (int64_t)e * E::PW + k);
+        for (int k = 0; k < E::M; ++k) s_row[E::PW + k] = __ldg(a.thr + (int64_t)e * E::M + k);
+    }
+    // site item
+    const uint32_t v = fdn.div(i), vc = c0 + (i - v * nc);
+    const bool has_site = i < nv && vc < C;
+    int64_t p0 = 0;
+    int deg = 0;
+    int code[KI];
+    if (has_site) { p0 = a.inc_ptr[v]; deg = (int)(a.inc_ptr[v + 1] - p0); }
 #pragma unroll
-                for (int x = 0; x < L; ++x) tot[x] = 0;
-                for (int c = 0; c < a.C; ++c) {
-                    const int x = xout[v * a.C + c];
+    for (int u = 0; u < KI; ++u) code[u] = u < deg ? __ldg(&a.inc[p0 + u].x) : -1;
+    float ut[L];
 #pragma unroll
-                    for (int y = 0; y < L; ++y) tot[y] += x == y ? 1u : 0u;
-                }
+    for (int x = 0; x < L; ++x) ut[x] = has_site ? __ldg(a.utf + (int64_t)v * L + x) : 0.0f;
+    if constexpr (S::KT > 0) {
 #pragma unroll
-                for (int x = 0; x < L; ++x) a.counts[v * L + x] += tot[x];
+        for (int u = 0; u < S::KT; ++u)
+            if (code[u] >= 0)
+                for (int k = 0; k < E::MP; ++k)
+                    s_row[S::TAU + u * E::MP + k] = __float_as_uint(__ldg(a.tau + (int64_t)(code[u] >> 1) * E::MP + k));
+    }
+    int lab = 0;
+    auto arrive = [&] { if (size > 1) cluster_arrive(); };
+    auto wait = [&] { if (size > 1) cluster_wait(); else __syncthreads(); };
+    arrive();
+    uint4 R[DualWords<L, LAYOUT>::N];
+    if (has_edge) draw_dual_words<L, LAYOUT>(e, ec, sweep, a.rk, R);
+    wait();                                                // labels in place; every CTA of the cluster has started
+    for (int it = 0; it < n_sweeps; ++it, ++sweep) {
+        if (has_edge) {
+            uint32_t bits[W];
+            const uint8_t* x = s_lab + (sweep & 1) * lab_bytes;
+            dual_bits<L, LAYOUT, false>(e, ec, x[ls], x[lt], s_row, s_row + E::PW, sweep, a.rk, bits, R);
+#pragma unroll
+            for (int w = 0; w < W; ++w) {
+                asm volatile("st.shared::cluster.u32 [%0],%1;" ::"r"(th_s + 4 * w), "r"(bits[w]) : "memory");
+                if (th_t != th_s) asm volatile("st.shared::cluster.u32 [%0],%1;" ::"r"(th_t + 4 * w), "r"(bits[w]) : "memory");
             }
         }
-        __syncthreads();
+        // the random words of the next half-step are drawn while the barrier completes
+        arrive();
+        float uni = 0.0f;
+        if (has_site) uni = uniform23(draw_rk(v, sweep, vc, PH_PRIMAL, 0, a.rk).x);
+        wait();
+        if (has_site) {
+            float acc[L], hi[L], lo[L];
+#pragma unroll
+            for (int x = 0; x < L; ++x) { acc[x] = 0.0f; hi[x] = 0.0f; lo[x] = 0.0f; }
+            int chunk = 0;
+            bool flushed = false;
+            auto words = [&](int cd, uint32_t (&bits)[W]) {
+                const uint32_t* th = s_th + ((uint32_t)(cd >> 1) * nc + (vc - c0)) * W;
+#pragma unroll
+                for (int w = 0; w < W; ++w) bits[w] = th[w];
+            };
+            auto flush = [&] {
+                if (++chunk == 32) {
+#pragma unroll
+                    for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], acc[x]); acc[x] = 0.0f; }
+                    chunk = 0;
+                    flushed = true;
+                }
+            };
+#pragma unroll
+            for (int u = 0; u < KI; ++u) {
+                if (code[u] < 0) continue;
+                uint32_t bits[W];
+                words(code[u], bits);
+                if constexpr (S::KT > 0)
+                    add_side<L, LAYOUT, false>(bits, reinterpret_cast<const float*>(s_row + S::TAU + u * E::MP), code[u] & 1, acc);
+                else
+                    add_side<L, LAYOUT>(bits, a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
+                flush();
+            }
+            for (int u = KI; u < deg; ++u) {
+                const int cd = __ldg(&a.inc[p0 + u].x);
+                uint32_t bits[W];
+                words(cd, bits);
+                add_side<L, LAYOUT>(bits, a.tau + (int64_t)(cd >> 1) * E::MP, cd & 1, acc);
+                flush();
+            }
+            float F[L];
+            if (flushed) {
+#pragma unroll
+                for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], acc[x]); F[x] = ut[x] + (hi[x] + lo[x]); }
+            } else {
+#pragma unroll
+                for (int x = 0; x < L; ++x) F[x] = ut[x] + acc[x];
+            }
+            float* lp = a.logp ? a.logp + ((int64_t)vc * a.N + v) * L : nullptr;
+            lab = draw_label_at<L>(F, uni, lp, a.ctl);
+            const uint32_t place = lab_addr + ((sweep + 1) & 1) * lab_bytes + i;
+            for (uint32_t r = 0; r < size; ++r)
+                asm volatile("st.shared::cluster.u8 [%0],%1;" ::"r"(cluster_address(place, r)), "r"(lab) : "memory");
+        }
+        arrive();
+        if (has_edge) draw_dual_words<L, LAYOUT>(e, ec, sweep + 1, a.rk, R);
+        if (has_site && sweep >= count_from) atomicAdd(a.counts + (int64_t)v * L + lab, 1u);
+        wait();
     }
-    if (threadIdx.x == 0) a.ctl->sweep = sweep;
+    if (has_site) a.x[(size_t)(sweep & 1) * a.N * a.C + (int64_t)v * C + vc] = (uint8_t)lab;
+    if (rank == 0 && threadIdx.x == 0) {                   // see k_sweep_small
+        __threadfence();
+        if (atomicAdd(&a.ctl->done, 1u) + 1u == gridDim.x / size) {
+            a.ctl->done = 0u;
+            a.ctl->sweep = sweep;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------- EM and mean field
@@ -1627,13 +1883,43 @@ cudaError_t run_mf(const SweepArgs& a, const float* qin, float* qout, cudaStream
 
 template <int L, int LAYOUT>
 cudaError_t run_sweep_small(const SweepArgs& a, int n_sweeps, cudaStream_t s) {
-    const size_t smem = (size_t)a.E * a.C * Ent<L, LAYOUT>::W * sizeof(uint32_t);
+    using S = SmallResident<L, LAYOUT>;
+    // Chains per cluster: at most two clusters per SM, at least 64 items each.  CTAs per cluster: a
+    // power of two, one item per thread and about 256 threads (64 and 128 measured the same, 512 and
+    // 1,024 slower: 100 sweeps of a 32 x 32 Ising grid 329 and 404 us against 300).  Models with more
+    // than 8 x 640 items per cluster, or more than 200 KB of tables per CTA, take k_sweep_small.
+    const int64_t per_chain = std::max<int64_t>(std::max<int64_t>(a.E, a.N), 1);
+    const int64_t nc = std::min<int64_t>(a.C, std::max<int64_t>((a.C + 303) / 304, (64 + per_chain - 1) / per_chain));
+    const int64_t items = per_chain * nc;
+    unsigned size = 1;
+    while (size < 8 && items > 256ll * size) size *= 2;
+    int64_t threads = ((items + size - 1) / size + 31) / 32 * 32;
+    int64_t smem = threads <= 640 ? S::smem(a.N * nc, a.E * nc, (int)threads) : 0;
+    const bool resident = threads <= 640 && smem <= 200 * 1024;
+    if (!resident) {
+        size = 1;
+        while (size < 8 && items > 512ll * size) size *= 2;
+        threads = 512;
+        smem = 0;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((a.C + nc - 1) / nc) * size);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = size;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = size > 1 ? 1 : 0;
+    if (!resident) return cudaLaunchKernelEx(&cfg, k_sweep_small<L, LAYOUT>, a, n_sweeps, FastDiv::make((uint32_t)nc));
     if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_sweep_small<L, LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(k_sweep_resident<L, LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_sweep_small<L, LAYOUT><<<1, 1024, smem, s>>>(a, n_sweeps);
-    return cudaGetLastError();
+    return cudaLaunchKernelEx(&cfg, k_sweep_resident<L, LAYOUT>, a, n_sweeps, FastDiv::make((uint32_t)nc));
 }
 
 template <int L, int LAYOUT>

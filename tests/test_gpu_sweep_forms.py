@@ -70,3 +70,43 @@ def test_sites_of_uneven_degree_match_the_oracle(L, C, E):
 @pytest.mark.parametrize("L,C", [(2, 64), (8, 64), (8, 5), (16, 32)])
 def test_label_draw_of_wide_fields_matches_the_oracle(L, C):
     _check(_wide_fields(L, 70 + L), C, 4000 + L)
+
+
+SMALL = {
+    "one_chain_L2": (lambda: wl.ising_grid(32, 32, seed=1), 1),                 # eight CTAs per cluster
+    "ten_chains_L2": (lambda: wl.ising_grid(50, 50, seed=2), 10),               # 640 threads per CTA
+    "too_many_items_per_chain": (lambda: wl.ising_grid(60, 70, seed=3), 5),     # more than 8 x 640
+    "tiny": (lambda: wl.tiny_random(3, 3, 2, seed=4), 1),
+    "single_site": (lambda: wl.Model(1, 5, np.zeros((1, 5), np.float32), np.zeros(0, np.int32), np.zeros(0, np.int32),
+                                     np.zeros((0, 5, 5), np.float32)), 3),
+    "several_chains_per_cluster": (lambda: wl.tiny_random(20, 4, 30, seed=5), 700),   # the last cluster is part full
+    "odd_chains": (lambda: wl.tiny_random(70, 3, 100, seed=6), 37),
+    "degree_79_L4": (lambda: wl.dense_potts(80, L=4, seed=7), 5),               # two-sum flushes
+    "wide_L16": (lambda: wl.random_graph(60, k=2, L=16, seed=8, w_std=0.3), 7), # table rows of 225 entries
+    "diag_L16": (lambda: wl.tiny_potts(90, 16, 200, seed=9), 9),
+    "lattice_L8": (lambda: wl.potts_grid3d(6, 6, 6, L=8, seed=10), 32),
+}
+
+
+@pytest.mark.parametrize("name", list(SMALL))
+def test_small_models_run_the_same_chain_in_one_launch(name):
+    make, C = SMALL[name]
+    model = make()
+    many, single = (make_handle(model, C, 77, schedule=1, use_graphs=False) for _ in range(2))
+    if model.n_edges > 3:                                  # free slots inside the edge list
+        for h in (many, single):
+            h.edit_factors(np.array([1, 3]), np.zeros(0, np.int32), np.zeros(0, np.int32),
+                           np.zeros((0, model.n_labels, model.n_labels), np.float32))
+            h.reset_marginals(2)
+    many.set_kernel_timing(True)
+    many.sweep(5)
+    assert list(many.kernel_times()) == ["k_sweep_small"]
+    for _ in range(5):
+        single.sweep(1)
+    assert np.array_equal(many.get_labels(), single.get_labels())
+    assert np.array_equal(many.counts(), single.counts())
+    assert many.boundary_draws() == single.boundary_draws()
+    for h in (many, single):                               # the sweep index advanced alike
+        h.sweep(1)
+    assert np.array_equal(many.get_labels(), single.get_labels())
+    assert many.info().sweep_index == single.info().sweep_index == 6
