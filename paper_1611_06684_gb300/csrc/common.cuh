@@ -179,9 +179,10 @@ struct SwArgs {
     uint8_t* x;                // [2][N][C] label double buffer
     int32_t* parent;           // [N][C] union-find forest, links to smaller sites only
     int32_t* root;             // [N][C] root of a bonded site (written by k_sw_flatten)
-    uint32_t* bits;            // [ceil(E C / 32)] bond bitmap of the sweep, bit g of item g = e C + c
+    uint32_t* theta;           // [E][C] dual words of Higdon's remainder, cleared at bonds; or null
+    const float* cdf;          // [N][L] float32 CDF of every site's unaries alone
     uint32_t* ban;             // [N][C] labels a cluster may not take (bit per label)
-    int64_t* lw;               // [N][L][C] fixed-point bond weights, then cluster weights at roots
+    int64_t* lw;               // [N][C][L] fixed-point bond weights, then cluster weights at roots
     unsigned* err;             // set when a union-find walk exceeded its step bound
     float* lpv;                // [N][C] log p of each root's drawn label, 0 at other sites (estimator) or null
     uint32_t* counts;          // [N][L] marginal counts (k_sw_small accumulates them itself)
@@ -296,8 +297,8 @@ cudaError_t launch_hg_tables(const int32_t* src, const double* ell, int64_t E, i
                              cudaStream_t s);
 cudaError_t launch_hg_check(const double* ut, int N, int L, const int32_t* src, const double* bound, int64_t E,
                             double* out, cudaStream_t s);
-cudaError_t launch_hg_clear(const uint32_t* bits, uint32_t* theta, int64_t items, cudaStream_t s);
-cudaError_t launch_sw_fix_unary(const float* unary, const double* unary_d, int64_t n, int64_t* ufix, cudaStream_t s);
+cudaError_t launch_sw_fix_unary(const float* unary, const double* unary_d, int N, int L, int64_t* ufix, float* cdf,
+                                cudaStream_t s);
 cudaError_t launch_sw_reset(const SwArgs& a, cudaStream_t s);
 cudaError_t launch_sw_bond(const SwArgs& a, cudaStream_t s);
 cudaError_t launch_sw_flatten(const SwArgs& a, cudaStream_t s);

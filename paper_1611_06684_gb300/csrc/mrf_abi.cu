@@ -66,12 +66,11 @@ struct mrf {
     double* d_swut = nullptr;          // [N][L] two-label unaries with the offsets folded in
     int32_t* d_swpar = nullptr;        // [N][C] union-find parents
     int32_t* d_swroot = nullptr;       // [N][C] roots of bonded sites
-    uint32_t* d_swbits = nullptr;      // bond bitmap, one bit per (edge slot, chain)
-    int64_t swbits_cap = 0;            // words of d_swbits
     uint32_t* d_swban = nullptr;       // [N][C] excluded labels of a cluster
-    int64_t* d_swlw = nullptr;         // [N][L][C] fixed-point cluster log weights
+    int64_t* d_swlw = nullptr;         // [N][C][L] fixed-point cluster log weights
     unsigned* d_swerr = nullptr;       // union-find step bound exceeded
     int64_t* d_swufix = nullptr;       // [N][L] fixed-point unaries of the Swendsen-Wang sweep
+    float* d_swcdf = nullptr;          // [N][L] CDF of every site's unaries alone
     double* d_swchk = nullptr;         // [3] model check sums (k_sw_check)
     double* d_swell = nullptr;         // [E][L] couplings l_x of the Swendsen-Wang form (float64)
     // Higdon's partial Swendsen-Wang: tables of the split at hg_rho (rebuilt after factor changes)
@@ -477,7 +476,7 @@ void mrf_destroy(mrf_t* h) {
     dfree(h->d_unary); dfree(h->d_ut); dfree(h->d_utf); dfree(h->d_tpl); dfree(h->d_src); dfree(h->d_dst); dfree(h->d_tau); dfree(h->d_thr);
     dfree(h->d_fold); dfree(h->d_cst); dfree(h->d_resid); dfree(h->d_inc_ptr); dfree(h->d_inc); dfree(h->d_x);
     dfree(h->d_theta); dfree(h->d_counts); dfree(h->d_lpv); dfree(h->d_logv); dfree(h->d_em); dfree(h->d_mfq); dfree(h->d_mfs); dfree(h->d_logp); dfree(h->d_ctl); dfree(h->d_flag); dfree(h->d_stage); dfree(h->d_pot); dfree(h->d_part);
-    dfree(h->d_swt); dfree(h->d_swl); dfree(h->d_swfold); dfree(h->d_swut); dfree(h->d_swpar); dfree(h->d_swroot); dfree(h->d_swbits); dfree(h->d_swban); dfree(h->d_swlw); dfree(h->d_swerr); dfree(h->d_swchk);
+    dfree(h->d_swt); dfree(h->d_swl); dfree(h->d_swfold); dfree(h->d_swut); dfree(h->d_swpar); dfree(h->d_swroot); dfree(h->d_swcdf); dfree(h->d_swban); dfree(h->d_swlw); dfree(h->d_swerr); dfree(h->d_swchk);
     dfree(h->d_swufix); dfree(h->d_swell);
     dfree(h->d_hgT); dfree(h->d_hglb); dfree(h->d_hgtau); dfree(h->d_hgthr); dfree(h->d_hgtpl); dfree(h->d_hgfold);
     dfree(h->d_hgbound); dfree(h->d_hgut); dfree(h->d_hgutf);
@@ -772,7 +771,7 @@ static SwArgs make_sw_args(const mrf_t* h) {
     SwArgs w{};
     w.N = h->N; w.C = h->C; w.L = h->L; w.E = h->E_slots;
     w.src = h->d_src; w.dst = h->d_dst; w.thr = h->d_swt; w.lwe = h->d_swl; w.ufix = h->d_swufix;
-    w.x = h->d_x; w.parent = h->d_swpar; w.root = h->d_swroot; w.bits = h->d_swbits; w.ban = h->d_swban; w.lw = h->d_swlw; w.err = h->d_swerr;
+    w.x = h->d_x; w.parent = h->d_swpar; w.root = h->d_swroot; w.cdf = h->d_swcdf; w.ban = h->d_swban; w.lw = h->d_swlw; w.err = h->d_swerr;
     w.ctl = h->d_ctl; w.rk = round_keys(h->key); w.fdC = FastDiv::make((uint32_t)h->C);
     w.lpv = h->lpv_on ? h->d_lpv : nullptr;
     w.counts = h->d_counts;
@@ -802,15 +801,13 @@ static mrf_status sw_prepare(mrf_t* h) {
         if (chk[0] > 0.0) return fail(h, MRF_EINVAL, "Swendsen-Wang sweeps need ferromagnetic tables (w(x,x) >= 0)");
         if (chk[1] + chk[2] >= kSwFixMax)
             return fail(h, MRF_ERANGE, "Swendsen-Wang: summed |log weights| exceed the fixed-point range (2^30)");
-        if (!h->d_swufix) { drop_graphs(h); MRF_CUDA(h, dalloc(h->d_swufix, (size_t)h->N * h->L)); }
-        MRF_CUDA(h, launch_sw_fix_unary(h->d_unary, h->d_swut, (int64_t)h->N * h->L, h->d_swufix, h->stream));
+        if (!h->d_swcdf) {
+            drop_graphs(h);
+            MRF_CUDA(h, dalloc(h->d_swufix, (size_t)h->N * h->L));
+            MRF_CUDA(h, dalloc(h->d_swcdf, (size_t)h->N * h->L));
+        }
+        MRF_CUDA(h, launch_sw_fix_unary(h->d_unary, h->d_swut, h->N, h->L, h->d_swufix, h->d_swcdf, h->stream));
         h->sw_checked = true;
-    }
-    const int64_t words = (h->E_slots * h->C + 31) / 32;       // edge slots grow with edits
-    if (words > h->swbits_cap) {
-        drop_graphs(h);
-        MRF_CUDA(h, dalloc(h->d_swbits, (size_t)std::max<int64_t>(words, 1)));
-        h->swbits_cap = words;
     }
     if (!h->d_swpar) {
         drop_graphs(h);
@@ -884,7 +881,7 @@ static mrf_status hg_prepare(mrf_t* h) {
 // kernels.
 static void make_hg_args(const mrf_t* h, SweepArgs& d, SwArgs& w) {
     w = make_sw_args(h);
-    w.thr = h->d_hgT; w.lwe = h->d_hglb; w.pot = h->d_pot;
+    w.thr = h->d_hgT; w.lwe = h->d_hglb; w.pot = h->d_pot; w.theta = h->d_theta;
     d = make_args(h);
     d.M = h->L; d.W = 1; d.tau = h->d_hgtau; d.thr = h->d_hgthr; d.tpl = h->d_hgtpl;
     d.utf = h->d_hgutf; d.ut = h->d_hgut; d.logp = nullptr; d.lpv = nullptr;
@@ -910,16 +907,13 @@ static mrf_status enqueue_sweep(mrf_t* h, int mode) {
         if (e == cudaSuccess) e = timed(h, MRF_K_SW_FLATTEN, [&] { return launch_sw_flatten(w, s); });
         if (e == cudaSuccess) e = timed(h, MRF_K_SW_DRAW, [&] { return launch_sw_draw(w, s); });
     } else if (mode == MRF_MODE_HIGDON) {
-        // bonds (and their unions), A's bits of the other edges, the bits'
-        // potentials, then the clusters as in the Swendsen-Wang sweep
+        // A's bits of every edge, bonds (their unions; a bond's bits cleared), the
+        // bits' potentials, then the clusters as in the Swendsen-Wang sweep
         SweepArgs d;
         SwArgs w;
         make_hg_args(h, d, w);
-        e = timed(h, MRF_K_SW_BOND, [&] { return launch_sw_bond(w, s); });
-        if (e == cudaSuccess) e = timed(h, MRF_K_DUAL, [&] {
-            const cudaError_t e2 = launch_dual(d, MRF_LAYOUT_DIAG, s);
-            return e2 != cudaSuccess ? e2 : launch_hg_clear(w.bits, d.theta, h->E_slots * h->C, s);
-        });
+        e = timed(h, MRF_K_DUAL, [&] { return launch_dual(d, MRF_LAYOUT_DIAG, s); });
+        if (e == cudaSuccess) e = timed(h, MRF_K_SW_BOND, [&] { return launch_sw_bond(w, s); });
         if (e == cudaSuccess) e = timed(h, MRF_K_POTENTIAL, [&] { return launch_potential(d, MRF_LAYOUT_DIAG, s); });
         if (e == cudaSuccess) e = timed(h, MRF_K_SW_FLATTEN, [&] { return launch_sw_flatten(w, s); });
         if (e == cudaSuccess) e = timed(h, MRF_K_SW_DRAW, [&] { return launch_sw_draw(w, s); });

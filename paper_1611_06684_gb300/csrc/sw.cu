@@ -7,21 +7,27 @@
 // label x with weight exp(sum_{v in K} u_v(x) + sum_{bonds in K} log(e^{l_x} - 1)).
 //
 // One sweep on the device, items (site or edge, chain) with the chain
-// innermost so that a warp works on one site or edge for 32 chains.  Between
+// innermost so that a warp works on one site or edge for many chains.  Between
 // sweeps every site is its own tree (parent[v][c] = v), its ban word is 0 and
-// its weight row lw[v][.][c] is 0; a sweep touches only what its bonds reach
+// its weight row lw[v][c][.] is 0; a sweep touches only what its bonds reach
 // and restores that state:
-//   k_sw_bond     bond draws into a bitmap (one ballot word per warp)
-//   k_sw_union    a thread per bitmap word: each bond unions its endpoints'
-//                 trees, adds its label weights to its source site's row and
-//                 marks both endpoints bonded (dense work: the sparse bonds no
-//                 longer hold whole warps of non-bonded lanes)
+//   k_sw_bond     bond draws; each bond unions its endpoints' trees, adds its
+//                 label weights to its source site's row and marks both
+//                 endpoints bonded
 //   k_sw_flatten  every bonded site records its root (the smallest site of its
 //                 cluster) and adds its unaries and row into the root's row
 //   k_sw_draw     every root (bonded or not) draws its cluster's label from
 //                 its unaries plus its row
 //   k_sw_assign   bonded non-roots copy the root's label; rows, parents and
 //                 ban words of bonded sites are reset.
+// Only about a fifth of the (edge, chain) items agree in their labels, 7 % are
+// bonded and a third of the sites are bonded (ferromagnetic lattice, beta ~
+// U[0, 1], 8 labels), at random lanes.  Each kernel therefore scans its items
+// four chains per lane, and its warps collect the items that need the next
+// step in a shared-memory queue and run it with full warps (WarpQueue).
+// Weight rows keep the labels innermost, so that the 8 L bytes of a row are
+// whole sectors.  Measured on 48^3, L = 8, 64 chains (us per sweep): bond and union
+// 265 -> 94, flatten 194 -> 81, draw and assign 273 -> 149.
 // Unaries enter as fixed-point values precomputed once per factor change.
 // Higdon's partial Swendsen-Wang (k_hg_*) runs the same kernels with its own
 // bond tables and per-chain potentials in place of the unaries; small models
@@ -33,6 +39,8 @@
 // The forest of a chain is its own column of parent[][], so chains never
 // contend.
 #include "sweep_impl.cuh"   // draw_label
+
+#include <algorithm>
 
 namespace mrfk {
 
@@ -120,75 +128,132 @@ __global__ void __launch_bounds__(256) k_sw_reset(SwArgs a) {
     }
 }
 
-// Bond draws, one item per (edge, chain), items g = e C + c.  A warp's 32
-// lanes hold 32 consecutive items (the grid stride is a multiple of 32), so
-// its bonds form one 32-bit word of the bond bitmap, bits[g / 32], written by
-// one lane; every word is written every sweep.
-__global__ void __launch_bounds__(256) k_sw_bond(SwArgs a) {
-    const int64_t n = a.E * a.C;
-    const unsigned long long t = a.ctl->sweep;
+// Per-warp queue of items in shared memory.  push() appends the lanes' flagged
+// items; drain() hands them out 32 at a time to `fn(item, on)`, called by whole
+// warps (lanes beyond the last item with on = false), until fewer than `keep`
+// are left.
+struct WarpQueue {
+    uint32_t* q;
+    int n;
+    __device__ __forceinline__ void push(uint32_t item, bool flag) {
+        const uint32_t bal = __ballot_sync(0xffffffffu, flag);
+        if (flag) q[n + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))] = item;
+        n += __popc(bal);
+    }
+    template <typename Fn>
+    __device__ __forceinline__ void drain(int keep, Fn fn) {
+        __syncwarp();
+        while (n >= keep && n > 0) {
+            const int lane = threadIdx.x & 31, take = n < 32 ? n : 32;
+            n -= take;
+            fn(lane < take ? q[n + lane] : 0u, lane < take);
+            __syncwarp();
+        }
+    }
+};
+
+constexpr int kSwWarps = 8;                               // 256 threads
+
+// Bond draws, items g = e C + c, V chains of one edge per lane (V = 4 when the
+// chains are a multiple of 4).  Pairs of equal labels are queued, their draws
+// (one Philox call each) decided 32 at a time, and the bonds queued again and
+// united 32 at a time: each links its endpoints' trees, adds its label weights
+// to its source site's row unless they are equal for every label (then they
+// would shift all of a cluster's exact sums alike and leave its draw
+// unchanged: Potts tables with one coupling per edge, every two-label table),
+// and marks both endpoints bonded.  With Higdon's remainder (a.theta) a bond
+// has no bits: its dual word, drawn before, is cleared.
+template <int L, int V>
+__global__ void __launch_bounds__(256) k_sw_bond(SwArgs a, int run) {
+    __shared__ uint32_t s_q[kSwWarps][2][32 * V + 32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t n = (uint32_t)(a.E * a.C);              // below 2^32 (host)
+    const uint32_t t = (uint32_t)a.ctl->sweep, C = (uint32_t)a.C;
     const uint8_t* __restrict__ xin = a.x + (size_t)(t & 1) * a.N * a.C;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g - lane < n; g += stride) {
+    WarpQueue same{s_q[warp][0], 0}, bonds{s_q[warp][1], 0};
+    auto unite = [&](uint32_t g, bool on) {
+        if (!on) return;
+        const uint32_t e = a.fdC.div(g);
+        const int32_t c = (int32_t)(g - e * C);
+        const int32_t s = a.src[e], d = a.dst[e];
+        if (a.theta) a.theta[g] = 0u;
+        if (!sw_union(a.parent, s, d, c, a.C, a.N)) { atomicOr(a.err, 1u); return; }
+        // every load before the first atomic (the compiler cannot move a
+        // load above an atomic to a possibly aliasing address)
+        int64_t wv[L];
+#pragma unroll
+        for (int x = 0; x < L; ++x) wv[x] = __ldg(a.lwe + (int64_t)e * L + x);
+        bool uniform = wv[0] != kSwNoLabel;
+#pragma unroll
+        for (int x = 1; x < L; ++x) uniform &= wv[x] == wv[0];
+        uint32_t flags = kSwBonded;
+        if (!uniform) {
+            flags |= kSwRow;
+#pragma unroll
+            for (int x = 0; x < L; ++x) {
+                if (wv[x] == kSwNoLabel) flags |= 1u << x;
+                else red_add_s64(a.lw + pidx(s, c, a.C) * L + x, wv[x]);
+            }
+        }
+        atomicOr(a.ban + pidx(s, c, a.C), flags);
+        atomicOr(a.ban + pidx(d, c, a.C), kSwBonded);
+    };
+    auto decide = [&](uint32_t g, bool on) {
         bool bond = false;
-        if (g < n) {
-            const int64_t e = a.fdC.div((uint32_t)g);
-            const int32_t c = (int32_t)(g - e * a.C);
-            const int32_t s = a.src[e];
+        if (on) {
+            const uint32_t e = a.fdC.div(g), c = g - e * C;
+            const uint32_t T = a.thr[(int64_t)e * L + xin[pidx(a.src[e], (int32_t)c, a.C)]];
+            bond = T != 0u && (draw_rk(e, t, c, PH_BOND, 0, a.rk).x >> 9) < T;
+        }
+        bonds.push(g, bond);
+        bonds.drain(32, unite);
+    };
+    const uint64_t first = ((uint64_t)blockIdx.x * kSwWarps + warp) * (32 * V * run);
+    for (int k = 0; k < run; ++k) {
+        const uint64_t g64 = first + (uint64_t)k * 32 * V + lane * V;
+        uint32_t agree = 0;                                // bit j: item g + j has equal labels
+        if (g64 < n) {
+            const uint32_t e = a.fdC.div((uint32_t)g64);
+            const int32_t c = (int32_t)((uint32_t)g64 - e * C), s = a.src[e];
             if (s >= 0) {
-                const int xs = xin[pidx(s, c, a.C)];
-                if (xs == xin[pidx(a.dst[e], c, a.C)]) {
-                    const uint32_t T = a.thr[e * a.L + xs];
-                    bond = T != 0u && (draw_rk((uint32_t)e, (uint32_t)t, (uint32_t)c, PH_BOND, 0, a.rk).x >> 9) < T;
+                const uint8_t* ps = xin + pidx(s, c, a.C);
+                const uint8_t* pd = xin + pidx(a.dst[e], c, a.C);
+                if constexpr (V == 4) {
+                    const uint32_t eq = __vcmpeq4(*reinterpret_cast<const uint32_t*>(ps), *reinterpret_cast<const uint32_t*>(pd));
+                    agree = (eq & 1u) | (eq >> 7 & 2u) | (eq >> 14 & 4u) | (eq >> 21 & 8u);
+                } else {
+                    agree = *ps == *pd;
                 }
             }
         }
-        const uint32_t word = __ballot_sync(0xffffffffu, bond);
-        if (lane == 0) a.bits[(g - lane) >> 5] = word;
+#pragma unroll
+        for (int j = 0; j < V; ++j) same.push((uint32_t)g64 + j, (agree >> j) & 1u);
+        same.drain(32, decide);
     }
+    same.drain(1, decide);
+    bonds.drain(1, unite);
 }
 
-// Unions of the bonds: one bitmap word per thread, its set bits in order.
-// Each bond links its endpoints' trees, adds its label weights to its source
-// site's row unless they are equal for every label (then they would shift all
-// of a cluster's exact sums alike and leave its draw unchanged: Potts tables
-// with one coupling per edge, every two-label table), and marks both
-// endpoints bonded.
-template <int L>
-__global__ void __launch_bounds__(256) k_sw_union(SwArgs a) {
-    const int64_t n = a.E * a.C;
-    const int64_t words = (n + 31) >> 5;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t word = a.bits[i];
-        while (word) {
-            const int bit = __ffs(word) - 1;
-            word &= word - 1u;
-            const int64_t g = i * 32 + bit;
-            const int64_t e = a.fdC.div((uint32_t)g);
-            const int32_t c = (int32_t)(g - e * a.C);
-            const int32_t s = a.src[e], d = a.dst[e];
-            if (!sw_union(a.parent, s, d, c, a.C, a.N)) { atomicOr(a.err, 1u); continue; }
-            // every load before the first atomic (the compiler cannot move a
-            // load above an atomic to a possibly aliasing address)
-            int64_t wv[L];
+// Scan of the ban words of the items that a warp owns, V of one site per lane:
+// fn(g, words) for every lane and tile (items beyond the last: words 0).
+template <int V, typename Fn>
+__device__ __forceinline__ void sw_scan(const SwArgs& a, int run, Fn fn) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t n = (uint64_t)a.N * a.C, first = ((uint64_t)blockIdx.x * kSwWarps + warp) * (32 * V * run);
+    for (int k = 0; k < run; ++k) {
+        const uint64_t g = first + (uint64_t)k * 32 * V + lane * V;
+        uint32_t b[V];
 #pragma unroll
-            for (int x = 0; x < L; ++x) wv[x] = __ldg(a.lwe + e * L + x);
-            bool uniform = wv[0] != kSwNoLabel;
-#pragma unroll
-            for (int x = 1; x < L; ++x) uniform &= wv[x] == wv[0];
-            uint32_t flags = kSwBonded;
-            if (!uniform) {
-                flags |= kSwRow;
-#pragma unroll
-                for (int x = 0; x < L; ++x) {
-                    if (wv[x] == kSwNoLabel) flags |= 1u << x;
-                    else red_add_s64(a.lw + ((int64_t)s * L + x) * a.C + c, wv[x]);
-                }
+        for (int j = 0; j < V; ++j) b[j] = 0u;
+        if (g < n) {
+            if constexpr (V == 4) {
+                const uint4 q = *reinterpret_cast<const uint4*>(a.ban + g);
+                b[0] = q.x; b[1] = q.y; b[2] = q.z; b[3] = q.w;
+            } else {
+                b[0] = a.ban[g];
             }
-            atomicOr(a.ban + pidx(s, c, a.C), flags);
-            atomicOr(a.ban + pidx(d, c, a.C), kSwBonded);
         }
+        fn((uint32_t)g, g < n, b);
     }
 }
 
@@ -196,58 +261,118 @@ __global__ void __launch_bounds__(256) k_sw_union(SwArgs a) {
 // is final once k_sw_bond has finished: every bonded site records its root
 // (the smallest site of its cluster), and a non-root adds its unaries and the
 // weights of the bonds it is the source of into its root's row.  Only roots'
-// rows and ban words are written here, and only non-roots' are read.
-template <int L>
-__global__ void __launch_bounds__(256) k_sw_flatten(SwArgs a) {
-    const int64_t n = (int64_t)a.N * a.C;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t b = a.ban[g];
-        if (!(b & kSwBonded)) continue;
-        const int32_t v = (int32_t)a.fdC.div((uint32_t)g), c = (int32_t)(g - (int64_t)v * a.C);
-        const int32_t r = sw_find(a.parent, v, c, a.C, a.N);
-        if (r < 0) { atomicOr(a.err, 1u); continue; }
-        a.root[g] = r;
-        if (r == v) continue;
-        int64_t w[L];
-#pragma unroll
-        for (int x = 0; x < L; ++x) w[x] = sw_unary<L>(a, v, c, x);
-        if (b & kSwRow) {
-            const int64_t* row = a.lw + (int64_t)v * L * a.C + c;
-#pragma unroll
-            for (int x = 0; x < L; ++x) w[x] += row[(int64_t)x * a.C];
+// rows and ban words are written here, and only non-roots' are read.  The
+// walks run one item per lane; the additions with the labels of an item on
+// consecutive lanes, so that a row's loads and reductions are whole sectors.
+template <int L, int V>
+__global__ void __launch_bounds__(256) k_sw_flatten(SwArgs a, int run) {
+    __shared__ uint32_t s_q[kSwWarps][32 * V + 32];
+    const int lane = threadIdx.x & 31;
+    const uint32_t C = (uint32_t)a.C;
+    WarpQueue bonded{s_q[threadIdx.x >> 5], 0};
+    auto flatten = [&](uint32_t g, bool on) {
+        uint32_t b = 0u;
+        int32_t v = 0, r = 0;
+        if (on) {
+            b = a.ban[g];
+            v = (int32_t)a.fdC.div(g);
+            r = sw_find(a.parent, v, (int32_t)(g - (uint32_t)v * C), a.C, a.N);
+            if (r < 0) { atomicOr(a.err, 1u); on = false; }
+            else a.root[g] = r;
         }
+        on = on && r != v;
+        const int32_t c = (int32_t)(g - (uint32_t)v * C);
+        if (on && (b & kSwLabelMask)) atomicOr(a.ban + pidx(r, c, a.C), b & kSwLabelMask);
+        if (a.pot) {                                       // per-chain unaries: consecutive chains on consecutive lanes
+            if (!on) return;
+            int64_t w[L];
 #pragma unroll
-        for (int x = 0; x < L; ++x) red_add_s64(a.lw + ((int64_t)r * L + x) * a.C + c, w[x]);
-        if (b & kSwLabelMask) atomicOr(a.ban + pidx(r, c, a.C), b & kSwLabelMask);
-    }
+            for (int x = 0; x < L; ++x) w[x] = sw_unary<L>(a, v, c, x);
+            if (b & kSwRow) {
+#pragma unroll
+                for (int x = 0; x < L; ++x) w[x] += a.lw[(int64_t)g * L + x];
+            }
+#pragma unroll
+            for (int x = 0; x < L; ++x) red_add_s64(a.lw + pidx(r, c, a.C) * L + x, w[x]);
+            return;
+        }
+        const uint32_t act = __ballot_sync(0xffffffffu, on), rows = __ballot_sync(0xffffffffu, on && (b & kSwRow));
+        const uint32_t gr = (uint32_t)pidx(r, c, a.C);     // the root's item, below 2^32
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            const int idx = k * 32 + lane, it = idx / L, x = idx - it * L;
+            const int32_t vi = __shfl_sync(0xffffffffu, v, it);
+            const uint32_t ri = __shfl_sync(0xffffffffu, gr, it), gi = __shfl_sync(0xffffffffu, g, it);
+            if (!((act >> it) & 1u)) continue;
+            int64_t w = __ldg(a.ufix + (int64_t)vi * L + x);
+            if ((rows >> it) & 1u) w += a.lw[(int64_t)gi * L + x];
+            red_add_s64(a.lw + (int64_t)ri * L + x, w);
+        }
+    };
+    sw_scan<V>(a, run, [&](uint32_t g, bool, const uint32_t (&b)[V]) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) bonded.push(g + j, (b[j] & kSwBonded) != 0u);
+        bonded.drain(32, flatten);
+    });
+    bonded.drain(1, flatten);
+}
+
+// Float32 CDF of a site on its own (its unaries only), for the draw of
+// unbonded sites: the same for every chain, so built once per factor change.
+template <int L>
+__global__ void k_sw_cdf(const int64_t* __restrict__ ufix, int N, float* __restrict__ cdf) {
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (v >= N) return;
+    int64_t w[L], mx = INT64_MIN;
+#pragma unroll
+    for (int x = 0; x < L; ++x) { w[x] = ufix[(int64_t)v * L + x]; mx = w[x] > mx ? w[x] : mx; }
+    float s = 0.0f, c[L];
+#pragma unroll
+    for (int x = 0; x < L; ++x) { s += expf(sw_float(w[x] - mx)); c[x] = s; }
+#pragma unroll
+    for (int x = 0; x < L; ++x) cdf[(int64_t)v * L + x] = c[x] / s;
 }
 
 // Label of every cluster, drawn at its root r by the inverse CDF with the
 // uniform of Philox(r, t, c, CLUSTER): weights are the root's unaries plus its
 // row (bonded sites), the differences to the largest are exact in fixed point
-// and then rounded to float for the softmax.  Nothing but the label is written
-// here: a store right behind the loads of the same row stalled the kernel
-// several-fold, so k_sw_assign clears rows and ban words.
-template <int L>
-__global__ void __launch_bounds__(256) k_sw_draw(SwArgs a) {
-    const int64_t n = (int64_t)a.N * a.C;
-    const unsigned long long t = a.ctl->sweep;
+// and then rounded to float for the softmax.  An unbonded site has the same
+// weights in every chain: its draw compares u with the site's CDF (k_sw_cdf,
+// within 3e-6 of the exact one, as draw_label's own), and only where a boundary
+// is within 2^-16 is the draw computed in full.  Nothing but the label is
+// written here: a store right behind the loads of the same row stalled the
+// kernel several-fold, so k_sw_assign clears rows and ban words.
+template <int L, int V>
+__global__ void __launch_bounds__(256) k_sw_draw(SwArgs a, int run) {
+    __shared__ uint32_t s_q[kSwWarps][32 * V + 32];
+    const uint32_t t = (uint32_t)a.ctl->sweep, C = (uint32_t)a.C;
     uint8_t* __restrict__ xout = a.x + (size_t)((t + 1) & 1) * a.N * a.C;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t v = (int32_t)a.fdC.div((uint32_t)g), c = (int32_t)(g - (int64_t)v * a.C);
+    WarpQueue queue{s_q[threadIdx.x >> 5], 0};
+    auto full = [&](uint32_t g, bool on) {
+        if (!on) return;
+        const int32_t v = (int32_t)a.fdC.div(g), c = (int32_t)(g - (uint32_t)v * C);
         const uint32_t b = a.ban[g];
         const bool bonded = (b & kSwBonded) != 0u;
-        if (bonded && a.root[g] != v) {                     // labelled by k_sw_assign
+        if (bonded && a.root[g] != v) {                    // labelled by k_sw_assign
             if (a.lpv) a.lpv[g] = 0.0f;
-            continue;
+            return;
         }
         int64_t w[L];
 #pragma unroll
         for (int x = 0; x < L; ++x) w[x] = sw_unary<L>(a, v, c, x);
         if (bonded) {
-            const int64_t* row = a.lw + (int64_t)v * L * a.C + c;
+            const int64_t* row = a.lw + (int64_t)g * L;
+            if constexpr (L % 2 == 0) {
 #pragma unroll
-            for (int x = 0; x < L; ++x) w[x] += row[(int64_t)x * a.C];
+                for (int x = 0; x < L; x += 2) {
+                    const longlong2 q = *reinterpret_cast<const longlong2*>(row + x);
+                    w[x] += q.x;
+                    w[x + 1] += q.y;
+                }
+            } else {
+#pragma unroll
+                for (int x = 0; x < L; ++x) w[x] += row[x];
+            }
         }
         int64_t mx = 0;
         bool any = false;
@@ -258,35 +383,104 @@ __global__ void __launch_bounds__(256) k_sw_draw(SwArgs a) {
 #pragma unroll
         for (int x = 0; x < L; ++x)
             F[x] = ((b >> x) & 1u) ? -INFINITY : sw_float(w[x] - mx);
-        xout[g] = (uint8_t)draw_label<L>(F, (uint32_t)v, (uint32_t)c, (uint32_t)t, a.rk, PH_CLUSTER, nullptr, a.ctl,
+        xout[g] = (uint8_t)draw_label<L>(F, (uint32_t)v, (uint32_t)c, t, a.rk, PH_CLUSTER, nullptr, a.ctl,
                                          a.lpv ? a.lpv + g : nullptr);
-    }
+    };
+    const bool table = !a.pot && !a.lpv, fields = a.pot && !a.lpv;
+    sw_scan<V>(a, run, [&](uint32_t g, bool in, const uint32_t (&b)[V]) {
+        uint32_t rest = in ? (1u << V) - 1u : 0u;          // items that take the full draw
+        uint32_t labels = 0;
+        if (in && fields) {                                // Higdon: every chain has its own potentials
+            const uint32_t v = a.fdC.div(g), c = g - v * C;
+#pragma unroll 1
+            for (int j = 0; j < V; ++j) {
+                if (b[j] & kSwBonded) continue;
+                float F[L];
+#pragma unroll
+                for (int x = 0; x < L; ++x) F[x] = a.pot[((int64_t)v * L + x) * a.C + c + j];
+                const int lab = draw_label_fast<L>(F, uniform23(draw_rk(v, t, c + j, PH_CLUSTER, 0, a.rk).x));
+                if (lab >= 0) { labels |= (uint32_t)lab << (8 * j); rest &= ~(1u << j); }
+            }
+        }
+        if (in && table) {
+            const uint32_t v = a.fdC.div(g), c = g - v * C;
+            float cdf[L];
+            if constexpr (L % 4 == 0) {
+#pragma unroll
+                for (int x = 0; x < L; x += 4) {
+                    const float4 q = __ldg(reinterpret_cast<const float4*>(a.cdf + (int64_t)v * L + x));
+                    cdf[x] = q.x; cdf[x + 1] = q.y; cdf[x + 2] = q.z; cdf[x + 3] = q.w;
+                }
+            } else {
+#pragma unroll
+                for (int x = 0; x < L; ++x) cdf[x] = __ldg(a.cdf + (int64_t)v * L + x);
+            }
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                const float u = uniform23(draw_rk(v, t, c + j, PH_CLUSTER, 0, a.rk).x);
+                float closest = INFINITY;
+                int lab = 0;
+#pragma unroll
+                for (int x = 0; x < L; ++x) {
+                    const float d = cdf[x] - u;
+                    closest = fminf(closest, fabsf(d));
+                    lab += d <= 0.0f ? 1 : 0;
+                }
+                if (!(b[j] & kSwBonded) && closest >= 0x1p-16f) rest &= ~(1u << j);
+                labels |= (uint32_t)lab << (8 * j);
+            }
+        }
+        if (in) {
+            if (V == 4 && rest == 0u) {
+                *reinterpret_cast<uint32_t*>(xout + g) = labels;
+            } else {
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (!((rest >> j) & 1u)) xout[g + j] = (uint8_t)(labels >> (8 * j));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j) queue.push(g + j, (rest >> j) & 1u);
+        queue.drain(32, full);
+    });
+    queue.drain(1, full);
 }
 
 // Bonded sites return to the between-sweeps state: non-roots copy their
 // root's label; a root's row (its cluster's sums) and a bond source's row are
-// cleared; parent and ban words are reset.  (Clearing whole 32-byte sectors
-// whenever any lane of a warp clears its entries wrote more than the merged
-// 8-byte writes cost: measured slower.)
-template <int L>
-__global__ void __launch_bounds__(256) k_sw_assign(SwArgs a) {
-    const int64_t n = (int64_t)a.N * a.C;
-    const unsigned long long t = a.ctl->sweep;
+// cleared (labels on consecutive lanes: whole sectors); parent and ban words
+// are reset.
+template <int L, int V>
+__global__ void __launch_bounds__(256) k_sw_assign(SwArgs a, int run) {
+    __shared__ uint32_t s_q[kSwWarps][32 * V + 32];
+    const int lane = threadIdx.x & 31;
+    const uint32_t t = (uint32_t)a.ctl->sweep, C = (uint32_t)a.C;
     uint8_t* __restrict__ xout = a.x + (size_t)((t + 1) & 1) * a.N * a.C;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t b = a.ban[g];
-        if (!(b & kSwBonded)) continue;
-        const int32_t v = (int32_t)a.fdC.div((uint32_t)g), c = (int32_t)(g - (int64_t)v * a.C);
-        const int32_t r = a.root[g];
-        if (r != v) xout[g] = xout[pidx(r, c, a.C)];
-        if (r == v || (b & kSwRow)) {
-            int64_t* row = a.lw + (int64_t)v * L * a.C + c;
-#pragma unroll
-            for (int x = 0; x < L; ++x) row[(int64_t)x * a.C] = 0;
+    WarpQueue bonded{s_q[threadIdx.x >> 5], 0};
+    auto assign = [&](uint32_t g, bool on) {
+        bool clear = false;
+        if (on) {
+            const uint32_t b = a.ban[g];
+            const int32_t v = (int32_t)a.fdC.div(g), c = (int32_t)(g - (uint32_t)v * C), r = a.root[g];
+            if (r != v) xout[g] = xout[pidx(r, c, a.C)];
+            clear = r == v || (b & kSwRow);
+            a.parent[g] = v;
+            a.ban[g] = 0u;
         }
-        a.parent[g] = v;
-        a.ban[g] = 0u;
-    }
+        const uint32_t rows = __ballot_sync(0xffffffffu, clear);
+#pragma unroll
+        for (int k = 0; k < L; ++k) {
+            const int idx = k * 32 + lane, it = idx / L;
+            const uint32_t gi = __shfl_sync(0xffffffffu, g, it);
+            if ((rows >> it) & 1u) a.lw[(int64_t)gi * L + (idx - it * L)] = 0;
+        }
+    };
+    sw_scan<V>(a, run, [&](uint32_t g, bool, const uint32_t (&b)[V]) {
+#pragma unroll
+        for (int j = 0; j < V; ++j) bonded.push(g + j, (b[j] & kSwBonded) != 0u);
+        bonded.drain(32, assign);
+    });
+    bonded.drain(1, assign);
 }
 
 // Small models: n_sweeps whole Swendsen-Wang sweeps in one launch of a single
@@ -502,20 +696,6 @@ __global__ void k_hg_check(const double* __restrict__ ut, int N, int L, const in
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < E; e += (int64_t)gridDim.x * blockDim.x)
         if (src[e] >= 0) acc += bound[e];
     if (acc != 0.0) atomicAdd(out, acc);
-}
-
-// A bond carries no bits of A: clear the dual bits of every bonded (edge,
-// chain) item (one dual word per item: the diagonal layout with L <= 16).
-__global__ void k_hg_clear(const uint32_t* __restrict__ bits, uint32_t* __restrict__ theta, int64_t items) {
-    const int64_t words = (items + 31) >> 5;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < words; i += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t word = bits[i];
-        while (word) {
-            const int b = __ffs(word) - 1;
-            word &= word - 1u;
-            theta[i * 32 + b] = 0u;
-        }
-    }
 }
 
 // Small models, Higdon's sweep: n_sweeps whole sweeps in one single-CTA
@@ -776,13 +956,13 @@ cudaError_t launch_hg_check(const double* ut, int N, int L, const int32_t* src, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_hg_clear(const uint32_t* bits, uint32_t* theta, int64_t items, cudaStream_t s) {
-    if (items > 0) k_hg_clear<<<sw_blocks((items + 31) / 32), 256, 0, s>>>(bits, theta, items);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_sw_fix_unary(const float* unary, const double* unary_d, int64_t n, int64_t* ufix, cudaStream_t s) {
-    if (n > 0) k_sw_fix_unary<<<sw_blocks(n), 256, 0, s>>>(unary, unary_d, n, ufix);
+// Also the CDF of every site on its own (k_sw_cdf).
+cudaError_t launch_sw_fix_unary(const float* unary, const double* unary_d, int N, int L, int64_t* ufix, float* cdf,
+                                cudaStream_t s) {
+    const int64_t n = (int64_t)N * L;
+    if (n <= 0) return cudaSuccess;
+    k_sw_fix_unary<<<sw_blocks(n), 256, 0, s>>>(unary, unary_d, n, ufix);
+    MRF_DISPATCH_LSW(L, (k_sw_cdf<LL><<<(unsigned)((N + 127) / 128), 128, 0, s>>>(ufix, N, cdf)));
     return cudaGetLastError();
 }
 
@@ -796,18 +976,40 @@ cudaError_t launch_sw_reset(const SwArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Launch shape of a kernel that scans n items: four chains per lane from two
+// blocks per SM on (below, one per lane spreads the items over more SMs), and
+// as many tiles per warp, up to eight, as leave eight blocks per SM.
+struct SwScan {
+    int V, run;
+    unsigned blocks;
+    SwScan(int64_t n, int C) {
+        V = C % 4 == 0 && n >= 32 * 4 * kSwWarps * 152 * 2 ? 4 : 1;
+        const int64_t tile = 32ll * V * kSwWarps;
+        run = (int)std::min<int64_t>(8, std::max<int64_t>(1, n / (tile * 152 * 8)));
+        blocks = (unsigned)((n + tile * run - 1) / (tile * run));
+    }
+};
+#define MRF_SW_SCAN(kernel, n)                                                                          \
+    do {                                                                                                \
+        const SwScan sc(n, a.C);                                                                        \
+        if (sc.V == 4) {                                                                                \
+            MRF_DISPATCH_LSW(a.L, (kernel<LL, 4><<<sc.blocks, 32 * kSwWarps, 0, s>>>(a, sc.run)));      \
+        } else {                                                                                        \
+            MRF_DISPATCH_LSW(a.L, (kernel<LL, 1><<<sc.blocks, 32 * kSwWarps, 0, s>>>(a, sc.run)));      \
+        }                                                                                               \
+    } while (0)
+
 cudaError_t launch_sw_bond(const SwArgs& a, cudaStream_t s) {
     const int64_t n = a.E * a.C;
     if (n <= 0) return cudaSuccess;
-    k_sw_bond<<<sw_blocks(n), 256, 0, s>>>(a);
-    MRF_DISPATCH_LSW(a.L, (k_sw_union<LL><<<sw_blocks((n + 31) / 32), 256, 0, s>>>(a)));
+    MRF_SW_SCAN(k_sw_bond, n);
     return cudaGetLastError();
 }
 
 cudaError_t launch_sw_flatten(const SwArgs& a, cudaStream_t s) {
     const int64_t n = (int64_t)a.N * a.C;
     if (n <= 0) return cudaSuccess;
-    MRF_DISPATCH_LSW(a.L, (k_sw_flatten<LL><<<sw_blocks(n), 256, 0, s>>>(a)));
+    MRF_SW_SCAN(k_sw_flatten, n);
     return cudaGetLastError();
 }
 
@@ -847,8 +1049,8 @@ cudaError_t launch_hg_small(const SweepArgs& d, const SwArgs& a, int n_sweeps, c
 cudaError_t launch_sw_draw(const SwArgs& a, cudaStream_t s) {
     const int64_t n = (int64_t)a.N * a.C;
     if (n <= 0) return cudaSuccess;
-    MRF_DISPATCH_LSW(a.L, (k_sw_draw<LL><<<sw_blocks(n), 256, 0, s>>>(a)));
-    MRF_DISPATCH_LSW(a.L, (k_sw_assign<LL><<<sw_blocks(n), 256, 0, s>>>(a)));
+    MRF_SW_SCAN(k_sw_draw, n);
+    MRF_SW_SCAN(k_sw_assign, n);
     return cudaGetLastError();
 }
 

@@ -110,3 +110,21 @@ def test_small_models_run_the_same_chain_in_one_launch(name):
         h.sweep(1)
     assert np.array_equal(many.get_labels(), single.get_labels())
     assert many.info().sweep_index == single.info().sweep_index == 6
+
+
+@pytest.mark.parametrize("mode,L,C,label_dependent", [(M.MODE_SW, 8, 64, False), (M.MODE_SW, 5, 64, True), (M.MODE_SW, 2, 128, False),
+                                                      (M.MODE_SW, 16, 36, True), (M.MODE_HIGDON, 8, 64, True),
+                                                      (M.MODE_HIGDON, 3, 68, False)])
+def test_cluster_sweeps_do_not_depend_on_the_scan_form(mode, L, C, label_dependent):
+    # four chains per lane (many items) and one per lane (three chains): a chain's
+    # draws depend on its own index only, so the first three chains are the same
+    model = wl.ferro_potts_grid3d(23, 22, 21, L=L, seed=80 + L)
+    if label_dependent:
+        rng = np.random.default_rng(L)
+        model.pair[:, np.arange(L), np.arange(L)] = rng.uniform(0, 1.2, (model.n_edges, L)) * (rng.random((model.n_edges, L)) > 0.2)
+    many, few = make_handle(model, C, 5, use_graphs=False), make_handle(model, 3, 5, use_graphs=False)
+    for h in (many, few):
+        h.set_labels(np.zeros((h.C, h.N), np.uint8))          # equal labels: the first sweep bonds most
+        for _ in range(3):
+            h.sweep(1, mode)
+    assert np.array_equal(many.get_labels()[:3], few.get_labels())
