@@ -110,6 +110,7 @@ struct SweepArgs {
     const float* resid;        // [E][L][L] exact tree-edge potentials (blocked sweep)
     const int64_t* inc_ptr;    // [N+1]
     int32_t max_deg;           // largest incidence count of a site (selects the primal kernels' one-batch form)
+    int32_t hub_deg;           // sites of more incidences are left to k_primal_hub (no limit: 0x7FFFFFFF)
     const int2* inc;           // [2E] {edge*2 + side, neighbour}
     const double* ut;          // [N][L] folded unaries
     uint8_t* x;                // [2][N][C] label double buffer
@@ -230,6 +231,11 @@ cudaError_t launch_primal(const SweepArgs& a, int layout, int schedule, cudaStre
 // Plain sweep in the edge-partial form (few chains, more than 16 entries per
 // edge), after the dual step: step 0 the per-edge partial fields, step 1 the labels.
 cudaError_t launch_sweep_partial(const SweepArgs& a, int layout, int step, cudaStream_t s);
+// Sites of more incidences than this are summed by a CTA each (k_primal_hub).
+// Preferential attachment, us per launch with a limit of 64 / 128 / 256 / none:
+// 50,000 sites, 32 chains 113 / 103 / 125 / 351; 10 chains 87 / 84 / 112 / 412;
+// 5,000 sites, 64 chains 45 / 59 / 90 / 95.
+constexpr int kHubDegree = 96;
 constexpr int kPartialMaxChains = 4;
 constexpr int kPartialMinEntries = 100;
 cudaError_t launch_fused(const SweepArgs& a, int layout, int schedule, cudaStream_t s);

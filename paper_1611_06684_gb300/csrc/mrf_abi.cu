@@ -180,7 +180,7 @@ SweepArgs make_args(const mrf_t* h) {
     a.E = h->E_slots;
     a.src = h->d_src; a.dst = h->d_dst; a.tau = h->d_tau; a.thr = h->d_thr; a.resid = h->d_resid;
     a.tpl = h->d_tpl; a.utf = h->d_utf;
-    a.inc_ptr = h->d_inc_ptr; a.inc = h->d_inc; a.ut = h->d_ut; a.max_deg = h->dyn_degree ? 0x7FFFFFFF : h->max_deg;
+    a.inc_ptr = h->d_inc_ptr; a.inc = h->d_inc; a.ut = h->d_ut; a.max_deg = h->dyn_degree ? 0x7FFFFFFF : h->max_deg; a.hub_deg = 0x7FFFFFFF;
     a.x = h->d_x; a.theta = h->d_theta; a.counts = h->d_counts; a.logp = h->d_logp;
     a.lpv = h->lpv_on ? h->d_lpv : nullptr;
     a.ctl = h->d_ctl; a.key = h->key;

@@ -643,6 +643,7 @@ __global__ void __launch_bounds__(256, FUSED ? 2 : 4) k_primal(SweepArgs a) {
     int xv = 0;
     if (FUSED) xv = xin[g];
     const int64_t p0 = a.inc_ptr[v], p1 = a.inc_ptr[v + 1];
+    if (!FUSED && p1 - p0 > a.hub_deg) return;                    // k_primal_hub's
     int chunk = 0;
     bool flushed = false;
     // Incidences in batches of B: all incidence records and (plain form) all
@@ -743,6 +744,7 @@ __global__ void __launch_bounds__(256, 4) k_primal_warp(SweepArgs a) {
     const uint32_t sweep = (uint32_t)a.ctl->sweep;
     uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
     const int64_t p0 = a.inc_ptr[v], p1 = a.inc_ptr[v + 1];
+    if (p1 - p0 > a.hub_deg) return;                              // k_primal_hub's
     const float4* tau4 = reinterpret_cast<const float4*>(a.tau);
     float F[L];
     const float* uf = a.utf + (int64_t)v * L;
@@ -1097,6 +1099,108 @@ __global__ void __launch_bounds__(128, PrimalPipe<L, LAYOUT, CH>::BLOCKS) k_prim
         __syncwarp();                                                    // this half is free for the unit after the next
         code = code1;
         code1 = code2;
+    }
+}
+
+// Sites of more than a.hub_deg incidences for the thread and warp forms above,
+// which would sum such a site in one thread or warp while the rest of the GPU
+// has finished (preferential attachment: a few sites of a thousand incidences
+// among 50,000).  A CTA looks through its share of the sites (spread so that
+// neighbouring hubs fall on different CTAs) and sums each hub with all its
+// threads: CG = min(C, 32) chains by 512 / CG slices, a slice one run of 32
+// incidences per round.  The forms above sum such a run from zero and then add
+// it to the site's two-sum pair; here the runs are summed side by side and added
+// to the pair in the same order, so the field is the same bit for bit.
+// 50,000 sites, 5 edges per new site (largest degree 1,548), L = 4, 32 chains:
+// potentials 355 -> 103 us; 10 chains 407 -> 84 us.
+template <int L, int LAYOUT, bool POT>
+__global__ void __launch_bounds__(512) k_primal_hub(SweepArgs a, int CG) {
+    using E = Ent<L, LAYOUT>;
+    constexpr int W = E::W, MAXH = 64;
+    __shared__ float s_part[L][512];
+    __shared__ int s_hub[MAXH];
+    __shared__ int s_n;
+    const int S = 512 / CG, lane = threadIdx.x % CG, slice = threadIdx.x / CG;
+    const uint32_t sweep = (uint32_t)a.ctl->sweep;
+    uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
+    for (int64_t v0 = blockIdx.x; v0 < a.N; v0 += (int64_t)gridDim.x * MAXH) {
+        __syncthreads();
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        for (int i = threadIdx.x; i < MAXH; i += 512) {
+            const int64_t v = v0 + (int64_t)i * gridDim.x;
+            if (v < a.N && a.inc_ptr[v + 1] - a.inc_ptr[v] > a.hub_deg) s_hub[atomicAdd(&s_n, 1)] = (int)v;
+        }
+        __syncthreads();
+        const int nh = s_n;
+        for (int q = 0; q < nh; ++q) {
+            const int v = s_hub[q];
+            const int64_t p0 = a.inc_ptr[v];
+            const int deg = (int)(a.inc_ptr[v + 1] - p0), runs = (deg + 31) / 32;
+            for (int cb = 0; cb < a.C; cb += CG) {
+                const int c = cb + lane;
+                float hi[L], lo[L], rest[L];
+#pragma unroll
+                for (int x = 0; x < L; ++x) { hi[x] = 0.0f; lo[x] = 0.0f; rest[x] = 0.0f; }
+                for (int r0 = 0; r0 < runs; r0 += S) {
+                    const int run = r0 + slice;
+                    if (slice < S && c < a.C && run < runs) {
+                        float acc[L];
+#pragma unroll
+                        for (int x = 0; x < L; ++x) acc[x] = 0.0f;
+                        const int end = min(deg, run * 32 + 32);
+                        constexpr int B = W <= 2 ? 4 : 2;  // incidences loaded together
+                        for (int u0 = run * 32; u0 < end; u0 += B) {
+                            int code[B];
+                            uint32_t bits[B][W];
+#pragma unroll
+                            for (int u = 0; u < B; ++u) code[u] = u0 + u < end ? __ldg(&a.inc[p0 + u0 + u].x) : -1;
+#pragma unroll
+                            for (int u = 0; u < B; ++u) {
+                                const uint32_t* th = a.theta + ((int64_t)(code[u] >> 1) * a.C + c) * W;
+#pragma unroll
+                                for (int w = 0; w < W; ++w) bits[u][w] = code[u] >= 0 ? __ldcs(th + w) : 0u;
+                            }
+#pragma unroll
+                            for (int u = 0; u < B; ++u)
+                                if (code[u] >= 0)
+                                    add_side<L, LAYOUT>(bits[u], a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
+                        }
+#pragma unroll
+                        for (int x = 0; x < L; ++x) s_part[x][threadIdx.x] = acc[x];
+                    }
+                    __syncthreads();
+                    if (slice == 0 && c < a.C) {
+                        for (int k = 0; k < S && r0 + k < runs; ++k) {
+                            if ((r0 + k) * 32 + 32 <= deg) {
+#pragma unroll
+                                for (int x = 0; x < L; ++x) two_sum_add(hi[x], lo[x], s_part[x][k * CG + lane]);
+                            } else {
+#pragma unroll
+                                for (int x = 0; x < L; ++x) rest[x] = s_part[x][k * CG + lane];
+                            }
+                        }
+                    }
+                    __syncthreads();
+                }
+                if (slice == 0 && c < a.C) {
+                    float F[L];
+                    const float* uf = a.utf + (int64_t)v * L;
+#pragma unroll
+                    for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], rest[x]); F[x] = __ldg(uf + x) + (hi[x] + lo[x]); }
+                    const int64_t g = (int64_t)v * a.C + c;
+                    if (POT) {
+                        float* pv = a.pot + (int64_t)v * L * a.C + c;
+#pragma unroll
+                        for (int x = 0; x < L; ++x) pv[(int64_t)x * a.C] = F[x];
+                    } else {
+                        float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
+                        xout[g] = (uint8_t)draw_label<L>(F, (uint32_t)v, (uint32_t)c, sweep, a.rk, PH_PRIMAL, lp, a.ctl,
+                                                         a.lpv ? a.lpv + g : nullptr);
+                    }
+                }
+            }
+        }
     }
 }
 
@@ -1849,23 +1953,39 @@ cudaError_t run_primal_warps(const SweepArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Thread or warp form of the plain primal step or its potentials.  A graph
+// with hubs leaves them to a second launch; where the largest degree may
+// change between launches (a batch's edit queue) there is none.
+template <int L, int LAYOUT, bool POT>
+cudaError_t run_field(const SweepArgs& args, cudaStream_t s) {
+    const int64_t n = (int64_t)args.N * args.C;
+    if (n <= 0) return cudaSuccess;
+    SweepArgs a = args;
+    const bool hubs = a.max_deg > kHubDegree && a.max_deg != 0x7FFFFFFF;
+    if (hubs) a.hub_deg = kHubDegree;
+    cudaError_t e = cudaSuccess;
+    if (a.C % 32 == 0) {
+        e = run_primal_warps<L, LAYOUT, POT>(a, s);
+    } else {
+        k_primal<L, LAYOUT, false, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
+        e = cudaGetLastError();
+    }
+    if (e != cudaSuccess || !hubs) return e;
+    const unsigned blocks = (unsigned)std::min<int64_t>(a.N, 152 * 2);
+    k_primal_hub<L, LAYOUT, POT><<<blocks, 512, 0, s>>>(a, std::min(a.C, 32));
+    return cudaGetLastError();
+}
+
 template <int L, int LAYOUT, bool FUSED>
 cudaError_t run_primal(const SweepArgs& a, cudaStream_t s) {
+    if constexpr (!FUSED) return run_field<L, LAYOUT, false>(a, s);
     const int64_t n = (int64_t)a.N * a.C;
-    if (n <= 0) return cudaSuccess;
-    if (!FUSED && a.C % 32 == 0) return run_primal_warps<L, LAYOUT, false>(a, s);
-    k_primal<L, LAYOUT, FUSED><<<blocks_for(n, 256), 256, 0, s>>>(a);
+    if (n > 0) k_primal<L, LAYOUT, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
     return cudaGetLastError();
 }
 
 template <int L, int LAYOUT>
-cudaError_t run_potential(const SweepArgs& a, cudaStream_t s) {
-    const int64_t n = (int64_t)a.N * a.C;
-    if (n <= 0) return cudaSuccess;
-    if (a.C % 32 == 0) return run_primal_warps<L, LAYOUT, true>(a, s);
-    k_primal<L, LAYOUT, false, true><<<blocks_for(n, 256), 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
+cudaError_t run_potential(const SweepArgs& a, cudaStream_t s) { return run_field<L, LAYOUT, true>(a, s); }
 
 template <int L, int LAYOUT>
 cudaError_t run_em(const SweepArgs& a, const uint8_t* xin, uint8_t* xout, cudaStream_t s) {

@@ -82,6 +82,12 @@ SMALL = {
     "several_chains_per_cluster": (lambda: wl.tiny_random(20, 4, 30, seed=5), 700),   # the last cluster is part full
     "odd_chains": (lambda: wl.tiny_random(70, 3, 100, seed=6), 37),
     "degree_79_L4": (lambda: wl.dense_potts(80, L=4, seed=7), 5),               # two-sum flushes
+    # sites of more than 96 incidences: one CTA each in the separate launches
+    "star_C32": (lambda: wl.Model(701, 3, np.random.default_rng(1).normal(size=(701, 3)).astype(np.float32),
+                                  np.zeros(700, np.int32), np.arange(1, 701, dtype=np.int32),
+                                  np.random.default_rng(2).normal(0, 0.3, (700, 3, 3)).astype(np.float32)), 32),
+    "dense_L3_C5": (lambda: wl.dense_potts(129, L=3, seed=11), 5),
+    "dense_L6_C1": (lambda: wl.dense_potts(161, L=6, seed=12), 1),
     "wide_L16": (lambda: wl.random_graph(60, k=2, L=16, seed=8, w_std=0.3), 7), # table rows of 225 entries
     "diag_L16": (lambda: wl.tiny_potts(90, 16, 200, seed=9), 9),
     "lattice_L8": (lambda: wl.potts_grid3d(6, 6, 6, L=8, seed=10), 32),
@@ -127,4 +133,16 @@ def test_cluster_sweeps_do_not_depend_on_the_scan_form(mode, L, C, label_depende
         h.set_labels(np.zeros((h.C, h.N), np.uint8))          # equal labels: the first sweep bonds most
         for _ in range(3):
             h.sweep(1, mode)
+    assert np.array_equal(many.get_labels()[:3], few.get_labels())
+
+
+@pytest.mark.parametrize("C", [64, 45])
+def test_hub_potentials_do_not_depend_on_the_chain_count(C):
+    # Higdon's potentials of a complete graph of 300 sites (299 incidences each): the hub CTAs'
+    # slices and rounds differ between 3 chains and C
+    model = wl.ferro_potts_graph(300, 4, 44850, beta_lo=0.0, beta_hi=0.02, seed=90)
+    many, few = make_handle(model, C, 6, use_graphs=False), make_handle(model, 3, 6, use_graphs=False)
+    for h in (many, few):
+        for _ in range(3):
+            h.sweep(1, M.MODE_HIGDON)
     assert np.array_equal(many.get_labels()[:3], few.get_labels())
