@@ -144,18 +144,17 @@ struct EntryDual {
     double alpha1, alpha2, log_norm;
 };
 //
-// With a = |l|, s = sqrt(1 - e^-a) and b = (1 + s)^2: tau = a + 2 log1p(s) and
-// e^-tau = e^-a / b, so sigmoid(+tau) = b / (b + e^-a), sigmoid(-tau) = e^-a / (b + e^-a)
-// and, for l > 0 (q = -tau), -log(1 + e^q) = -log1p(e^-a / b): four float64
-// transcendentals per entry (expm1, exp, two log1p) and one division.
+// With a = |l| and s = sqrt(1 - e^-a): tau = a + 2 log1p(s); e^-tau = e^-a / (1 + s)^2
+// and e^-a = (1 - s)(1 + s), so sigmoid(+tau) = (1 + s) / 2 and sigmoid(-tau) = (1 - s) / 2,
+// and for l > 0 (q = -tau) -log(1 + e^q) = log sigmoid(tau) = log1p(s) - log 2: two float64
+// transcendentals and a square root per entry, which is what the decomposition's time
+// is (GB300's float64 rate).
 __host__ __device__ inline EntryDual entry_dual(double l) {
     const double al = fabs(l);
-    const double s = sqrt(-expm1(-al));
-    const double tau = al + 2.0 * log1p(s);
-    const double ea = exp(-al), b = (1.0 + s) * (1.0 + s);
-    const double inv = 1.0 / (b + ea);
-    const double pp = b * inv;                   // sigmoid(+tau)
-    const double pm = ea * inv;                  // sigmoid(-tau)
+    const double s = sqrt(-expm1(-al)), g = log1p(s);
+    const double tau = al + 2.0 * g;
+    const double pp = 0.5 * (1.0 + s);           // sigmoid(+tau)
+    const double pm = 0.5 * (1.0 - s);           // sigmoid(-tau)
     const uint32_t tp = (uint32_t)ceil(pp * 16777216.0 - 0.5), tm = (uint32_t)ceil(pm * 16777216.0 - 0.5);
     const uint32_t d = tp + tm - ((1u << 24) - 1u);   // in {0,1,2}
     EntryDual r;
@@ -163,7 +162,7 @@ __host__ __device__ inline EntryDual entry_dual(double l) {
     r.tau_s = (float)(l > 0 ? tau : -tau);
     r.alpha1 = l > 0 ? 0.5 * (l - tau) : 0.5 * (l + tau);
     r.alpha2 = 0.5 * (l - tau);
-    r.log_norm = l > 0 ? -log1p(ea / b) : -0.69314718055994530942;   // q = -tau, or q = 0: -log 2
+    r.log_norm = l > 0 ? g - 0.69314718055994530942 : -0.69314718055994530942;   // q = -tau, or q = 0: -log 2
     return r;
 }
 

@@ -21,6 +21,7 @@
 // exactly u = (U + 1/2) / 2^24 < p.  All of this runs in float64.
 #include "common.cuh"
 
+#include <algorithm>
 #include <cmath>
 
 namespace mrfk {
@@ -32,64 +33,91 @@ __global__ void k_check_finite(const float* p, int64_t n, unsigned long long* ba
     if (cnt) atomicAdd(bad, cnt);
 }
 
-__global__ void k_count_offdiag(const float* pair, int64_t n_edges, int L, unsigned long long* nz) {
-    const int64_t n = n_edges * L * L;
+// One row of a table per thread, one atomic per block (one per thread held
+// every table with off-diagonal values up on a single address: 153,040 tables of
+// 5 x 5 took 209 us for 15 MB).
+__global__ void k_count_offdiag(const float* pair, int64_t n_edges, int L, FastDiv fdL, unsigned long long* nz) {
+    const int64_t rows = n_edges * L;
     unsigned long long cnt = 0;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int r = (int)((i / L) % L), c = (int)(i % L);
-        cnt += (r != c) && (pair[i] != 0.0f);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < rows; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t e0 = i < 0xFFFFFFFFll ? (int64_t)fdL.div((uint32_t)i) : i / L;
+        const int r = (int)(i - e0 * L);
+        for (int c = 0; c < L; ++c) cnt += (r != c) && (pair[i * L + c] != 0.0f);
     }
-    if (cnt) atomicAdd(nz, cnt);
+    __shared__ unsigned long long s_cnt;
+    if (threadIdx.x == 0) s_cnt = 0ull;
+    __syncthreads();
+    cnt = __reduce_add_sync(0xffffffffu, (unsigned)cnt);   // a thread's share is far below 2^27
+    if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(&s_cnt, cnt);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_cnt) atomicAdd(nz, s_cnt);
 }
 
-__global__ void k_decompose(DecompArgs a) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= a.n || (a.n_dev && i >= *a.n_dev) || (a.status && (*a.status & kQFatal))) return;
-    const int L = a.L, M = a.M;
-    const int64_t e = a.slots ? a.slots[i] : a.first_slot + i;
-    const float* w = a.pair + (a.pair_off ? a.pair_off[i] : i * L * L);
-    double fs[kMaxLabels], ft[kMaxLabels];
-    double cst = 0.0;
-    if (a.layout == MRF_LAYOUT_PIVOT) {
-        const double w00 = w[0];
-        for (int x = 0; x < L; ++x) {
-            fs[x] = (double)w[x * L] - w00;
-            ft[x] = (double)w[x] - w00;
-        }
-        cst = w00;
-    } else {
-        for (int x = 0; x < L; ++x) fs[x] = ft[x] = 0.0;
-    }
-    for (int k = 0; k < M; ++k) {
-        int ii, jj;
+// A block takes `eb` edges.  Their entries are spread over its threads (the
+// float64 transcendentals of entry_dual are the kernel's time, so every lane
+// has one, and few edges still fill the GPU: 1,470 new edges of 225 entries in
+// a thread per edge took 1.53 ms, 0.16 ms here); the entries' terms meet in
+// shared memory, where a thread per row or column sums them in entry order.
+constexpr int kDecompItems = 512;                          // entries of a block
+__global__ void __launch_bounds__(128) k_decompose(DecompArgs a, int eb) {
+    __shared__ double s_a1[kDecompItems], s_a2[kDecompItems], s_ln[kDecompItems];
+    __shared__ double s_f[kDecompItems * 2];               // folded rows and columns of the block's edges
+    __shared__ double s_row[kDecompItems];             // log-constant terms per row
+    const int64_t n = a.n_dev && *a.n_dev < a.n ? *a.n_dev : a.n;
+    const int64_t i0 = (int64_t)blockIdx.x * eb;
+    if (i0 >= n || (a.status && (*a.status & kQFatal))) return;
+    const int L = a.L, M = a.M, MP = pad4(M), ne = (int)(n - i0 < eb ? n - i0 : eb), tid = threadIdx.x;
+    const bool pivot = a.layout == MRF_LAYOUT_PIVOT;
+    auto slot = [&](int q) { return a.slots ? a.slots[i0 + q] : a.first_slot + i0 + q; };
+    auto table = [&](int q) { return a.pair + (a.pair_off ? a.pair_off[i0 + q] : (i0 + q) * L * L); };
+    for (int it = tid; it < ne * M; it += 128) {
+        const int q = it / M, k = it - q * M;
+        const float* w = table(q);
         double l;
-        if (a.layout == MRF_LAYOUT_PIVOT) {
-            ii = 1 + k / (L - 1); jj = 1 + k % (L - 1);
+        if (pivot) {
+            const int r = k / (L - 1), ii = 1 + r, jj = 1 + k - r * (L - 1);
             l = (double)w[ii * L + jj] - (double)w[ii * L] - (double)w[jj] + (double)w[0];
         } else {
-            ii = jj = k;
             l = (double)w[k * L + k];
         }
-        float tau_s = 0.0f;
-        uint32_t word = 0;
-        if (l != 0.0) {
-            const EntryDual d = entry_dual(l);
-            word = d.word;
-            tau_s = d.tau_s;
-            fs[ii] += d.alpha1;
-            ft[jj] += d.alpha2;
-            cst += d.log_norm;   // -log(1 + e^q)
+        EntryDual d{};
+        if (l != 0.0) d = entry_dual(l);
+        s_a1[it] = d.alpha1; s_a2[it] = d.alpha2; s_ln[it] = d.log_norm;   // -log(1 + e^q)
+        const int64_t e = slot(q);
+        a.tau[e * MP + k] = d.tau_s;
+        a.thr[e * M + k] = d.word;
+        if (k < MP - M) a.tau[e * MP + M + k] = 0.0f;      // the row's padding (at most 3, M = 1: see below)
+        if (M == 1) { a.tau[e * MP + 2] = 0.0f; a.tau[e * MP + 3] = 0.0f; }
+    }
+    __syncthreads();
+    // entries of row x (source side) or column x (destination side), in entry order
+    for (int j = tid; j < ne * 2 * L; j += 128) {
+        const int q = j / (2 * L), sd = j - q * 2 * L, side = sd >= L, x = sd - side * L;
+        const float* w = table(q);
+        double f = 0.0, ln = 0.0;
+        if (pivot) {
+            f = (double)w[side ? x : x * L] - (double)w[0];
+            if (x > 0)
+                for (int y = 0; y < L - 1; ++y) {
+                    const int k = q * M + (side ? y * (L - 1) + x - 1 : (x - 1) * (L - 1) + y);
+                    f += side ? s_a2[k] : s_a1[k];
+                    if (!side) ln += s_ln[k];
+                }
+        } else {
+            f += side ? s_a2[q * M + x] : s_a1[q * M + x];
+            ln = s_ln[q * M + x];
         }
-        a.tau[e * pad4(M) + k] = tau_s;
-        a.thr[e * M + k] = word;
+        s_f[j] = f;
+        if (!side) s_row[q * L + x] = ln;
+        a.fold[slot(q) * 2 * L + sd] = f;
     }
-    for (int k = M; k < pad4(M); ++k) a.tau[e * pad4(M) + k] = 0.0f;
-    for (int x = 0; x < L; ++x) {
-        a.fold[(e * 2 + 0) * L + x] = fs[x];
-        a.fold[(e * 2 + 1) * L + x] = ft[x];
+    __syncthreads();
+    for (int q = tid; q < ne; q += 128) {
+        double cst = pivot ? (double)table(q)[0] : 0.0;
+        for (int x = 0; x < L; ++x) cst += s_row[q * L + x];
+        a.cst[slot(q)] = cst;
     }
-    a.cst[e] = cst;
-    if (a.sw_thr && (a.layout == MRF_LAYOUT_DIAG || L == 2)) {
+    if (a.sw_thr && (!pivot || L == 2)) {
         // Swendsen-Wang tables (Section 4.3): the table as
         // c + f(a) + g(b) + l_a [a = b] -- diagonal tables: l_x = w(x,x), f = g = 0;
         // two labels: l = (w00 + w11 - w01 - w10) / 2 for both labels,
@@ -98,21 +126,20 @@ __global__ void k_decompose(DecompArgs a) {
         // T = ceil(p 2^23 - 1/2) (a draw U bonds iff U < T, i.e. (U + 1/2) / 2^23 < p),
         // and the bond's label weight log(e^{l_x} - 1) in fixed point (sw_fix);
         // l <= 0: no bond (T = 0) and the label is excluded when bonded (kSwNoLabel).
-        double lx[kMaxLabels];
-        if (L == 2) {
-            const double k2 = 0.5 * ((double)w[0] + (double)w[3] - (double)w[1] - (double)w[2]);
-            lx[0] = lx[1] = k2;
-            if (a.sw_fold) {
-                a.sw_fold[(e * 2 + 0) * 2 + 0] = 0.0;
-                a.sw_fold[(e * 2 + 0) * 2 + 1] = (double)w[2] - (double)w[0] + k2;
-                a.sw_fold[(e * 2 + 1) * 2 + 0] = 0.0;
-                a.sw_fold[(e * 2 + 1) * 2 + 1] = (double)w[1] - (double)w[0] + k2;
+        for (int j = tid; j < ne * L; j += 128) {
+            const int q = j / L, x = j - q * L;
+            const float* w = table(q);
+            const int64_t e = slot(q);
+            double l;
+            if (L == 2) {
+                l = 0.5 * ((double)w[0] + (double)w[3] - (double)w[1] - (double)w[2]);
+                if (a.sw_fold) {
+                    a.sw_fold[(e * 2 + 0) * 2 + x] = x ? (double)w[2] - (double)w[0] + l : 0.0;
+                    a.sw_fold[(e * 2 + 1) * 2 + x] = x ? (double)w[1] - (double)w[0] + l : 0.0;
+                }
+            } else {
+                l = (double)w[x * L + x];
             }
-        } else {
-            for (int x = 0; x < L; ++x) lx[x] = (double)w[x * L + x];
-        }
-        for (int x = 0; x < L; ++x) {
-            const double l = lx[x];
             uint32_t T = 0;
             int64_t lw = kSwNoLabel;
             if (l > 0.0) {
@@ -127,9 +154,11 @@ __global__ void k_decompose(DecompArgs a) {
     if (a.resid) {
         // exact pairwise potential in the folded representation (tree edges of
         // the blocked sweep): w(a,b) - fold_s(a) - fold_t(b)
-        for (int x = 0; x < L; ++x)
-            for (int y = 0; y < L; ++y)
-                a.resid[(e * L + x) * L + y] = (float)((double)w[x * L + y] - fs[x] - ft[y]);
+        for (int j = tid; j < ne * L * L; j += 128) {
+            const int q = j / (L * L), xy = j - q * L * L, x = xy / L, y = xy - x * L;
+            a.resid[slot(q) * L * L + xy] =
+                (float)((double)table(q)[xy] - s_f[q * 2 * L + x] - s_f[q * 2 * L + L + y]);
+        }
     }
 }
 
@@ -182,22 +211,17 @@ __global__ void k_build_planes(const uint32_t* thr, int64_t n, const int64_t* sl
     out[4] = make_uint4(S, Act, 0u, 0u);
 }
 
+// A thread per (site, label): the incidences' terms in order, float64.
 __global__ void k_fold_unary(const float* unary, const double* unary_d, const double* fold, const int64_t* inc_ptr,
-                             const int2* inc, int N, int L, double* ut, float* utf) {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= N) return;
-    double acc[kMaxLabels];
-    for (int x = 0; x < L; ++x) acc[x] = unary_d ? unary_d[(int64_t)v * L + x] : (double)unary[(int64_t)v * L + x];
-    for (int64_t p = inc_ptr[v]; p < inc_ptr[v + 1]; ++p) {
-        const int code = inc[p].x;
-        const int64_t e = code >> 1;
-        const double* f = fold + (e * 2 + (code & 1)) * L;
-        for (int x = 0; x < L; ++x) acc[x] += f[x];
-    }
-    for (int x = 0; x < L; ++x) {
-        ut[(int64_t)v * L + x] = acc[x];
-        if (utf) utf[(int64_t)v * L + x] = (float)acc[x];
-    }
+                             const int2* inc, int N, int L, FastDiv fdL, double* ut, float* utf) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= (int64_t)N * L) return;
+    const int64_t v = i < 0xFFFFFFFFll ? (int64_t)fdL.div((uint32_t)i) : i / L;
+    const int x = (int)(i - v * L);
+    double acc = unary_d ? unary_d[i] : (double)unary[i];
+    for (int64_t p = inc_ptr[v]; p < inc_ptr[v + 1]; ++p) acc += fold[(int64_t)inc[p].x * L + x];   // code = 2 edge + side
+    ut[i] = acc;
+    if (utf) utf[i] = (float)acc;
 }
 
 cudaError_t launch_check_finite(const float* p, int64_t n, unsigned long long* bad, cudaStream_t s) {
@@ -206,18 +230,25 @@ cudaError_t launch_check_finite(const float* p, int64_t n, unsigned long long* b
 }
 
 cudaError_t launch_count_offdiag(const float* pair, int64_t n_edges, int L, unsigned long long* nz, cudaStream_t s) {
-    if (n_edges > 0) k_count_offdiag<<<1216, 256, 0, s>>>(pair, n_edges, L, nz);
+    if (n_edges > 0) k_count_offdiag<<<1216, 256, 0, s>>>(pair, n_edges, L, FastDiv::make((uint32_t)L), nz);
     return cudaGetLastError();
 }
 
 cudaError_t launch_decompose(const DecompArgs& a, cudaStream_t s) {
-    if (a.n > 0) k_decompose<<<(unsigned)((a.n + 127) / 128), 128, 0, s>>>(a);
+    if (a.n <= 0) return cudaSuccess;
+    // up to 512 entries (and 512 row sums) per block, fewer while the blocks do not fill the GPU
+    const int most = std::max(1, kDecompItems / std::max(a.M, a.L));
+    const int eb = (int)std::min<int64_t>(most, std::max<int64_t>(std::max(1, 128 / a.M), (a.n + 152 * 8 - 1) / (152 * 8)));
+    k_decompose<<<(unsigned)((a.n + eb - 1) / eb), 128, 0, s>>>(a, eb);
     return cudaGetLastError();
 }
 
 cudaError_t launch_fold_unary(const float* unary, const double* fold, const int64_t* inc_ptr, const int2* inc,
                               int N, int L, double* ut, float* utf, cudaStream_t s, const double* unary_d) {
-    if (N > 0) k_fold_unary<<<(N + 127) / 128, 128, 0, s>>>(unary, unary_d, fold, inc_ptr, inc, N, L, ut, utf);
+    const int64_t n = (int64_t)N * L;
+    if (n > 0)
+        k_fold_unary<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(unary, unary_d, fold, inc_ptr, inc, N, L,
+                                                                 FastDiv::make((uint32_t)L), ut, utf);
     return cudaGetLastError();
 }
 

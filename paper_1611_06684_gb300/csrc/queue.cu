@@ -292,22 +292,20 @@ __global__ void k_q_place(QClass c, int64_t cap, int64_t* out_slot, uint32_t* st
 
 // Folded unaries (Sections 4.1-4.2 offsets of every incident edge) of the
 // sites an edit touched, in incidence order as in the full fold.
-__global__ void k_fold_touched(const float* unary, const double* fold, const int64_t* inc_ptr, const int2* inc,
-                               int N, int L, uint8_t* touched, double* ut, float* utf) {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= N || !touched[v]) return;
-    touched[v] = 0;
-    double acc[kMaxLabels];
-    for (int x = 0; x < L; ++x) acc[x] = (double)unary[(int64_t)v * L + x];
-    for (int64_t p = inc_ptr[v]; p < inc_ptr[v + 1]; ++p) {
-        const int code = inc[p].x;
-        const double* f = fold + ((int64_t)(code >> 1) * 2 + (code & 1)) * L;
-        for (int x = 0; x < L; ++x) acc[x] += f[x];
-    }
-    for (int x = 0; x < L; ++x) {
-        ut[(int64_t)v * L + x] = acc[x];
-        utf[(int64_t)v * L + x] = (float)acc[x];
-    }
+__global__ void __launch_bounds__(256) k_fold_touched(const float* unary, const double* fold, const int64_t* inc_ptr,
+                                                      const int2* inc, int N, int L, uint8_t* touched, double* ut,
+                                                      float* utf) {
+    // a thread per (site, label); a block owns whole sites, so that a mark is cleared after all have read it
+    const int sites = 256 / L, vl = threadIdx.x / L, x = threadIdx.x - vl * L;
+    const int64_t v = (int64_t)blockIdx.x * sites + vl;
+    const bool mine = vl < sites && v < N && touched[v];
+    __syncthreads();
+    if (!mine) return;
+    if (x == 0) touched[v] = 0;
+    double acc = (double)unary[v * L + x];
+    for (int64_t p = inc_ptr[v]; p < inc_ptr[v + 1]; ++p) acc += fold[(int64_t)inc[p].x * L + x];   // code = 2 edge + side
+    ut[v * L + x] = acc;
+    utf[v * L + x] = (float)acc;
 }
 
 __global__ void k_q_finish(QArgs q) {
@@ -376,7 +374,8 @@ cudaError_t launch_queue_apply(const QArgs& q, const QClass& c, cudaStream_t s) 
 
 cudaError_t launch_fold_touched(const float* unary, const double* fold, const int64_t* inc_ptr, const int2* inc,
                                 int N, int L, uint8_t* touched, double* ut, float* utf, cudaStream_t s) {
-    if (N > 0) k_fold_touched<<<(N + 255) / 256, 256, 0, s>>>(unary, fold, inc_ptr, inc, N, L, touched, ut, utf);
+    const int sites = 256 / L;
+    if (N > 0) k_fold_touched<<<(N + sites - 1) / sites, 256, 0, s>>>(unary, fold, inc_ptr, inc, N, L, touched, ut, utf);
     return cudaGetLastError();
 }
 
