@@ -56,7 +56,7 @@ __global__ void k_count_offdiag(const float* pair, int64_t n_edges, int L, FastD
 // A block takes `eb` edges.  Their entries are spread over its threads (the
 // float64 transcendentals of entry_dual are the kernel's time, so every lane
 // has one, and few edges still fill the GPU: 1,470 new edges of 225 entries in
-// a thread per edge took 1.53 ms, 0.16 ms here); the entries' terms meet in
+// a thread per edge took 1.53 ms, 0.10 ms here); the entries' terms meet in
 // shared memory, where a thread per row or column sums them in entry order.
 constexpr int kDecompItems = 512;                          // entries of a block
 __global__ void __launch_bounds__(128) k_decompose(DecompArgs a, int eb) {

@@ -387,6 +387,9 @@ __device__ __forceinline__ int draw_label(const float (&F)[L], uint32_t v, uint3
 // decides the queued entries with one entry per lane per round and ORs the
 // won bits into the staged words, which are then stored.  Ties of a lane
 // whose entry does not fit the queue are decided by the lane itself.
+// PART: ng < NG groups per warp, where NG would leave SMs without a block
+// (run_dual); an instance of its own, for the loop bound's sake (a variable
+// bound for all cost 9 % on 447,262 edges of L = 5, 24 chains).
 template <int M, int W>
 struct DualTile {
     static constexpr int WARPS = 8;                                         // 256 threads
@@ -397,23 +400,24 @@ struct DualTile {
 };
 
 // FEW: the launch bounds of the form for fewer than 32 chains (run_dual).
-template <int L, int LAYOUT, bool FEW = false>
-__global__ void __launch_bounds__(256, FEW ? 2 : 4) k_dual(SweepArgs a) {
+template <int L, int LAYOUT, bool FEW = false, bool PART = false>
+__global__ void __launch_bounds__(256, FEW ? 2 : 4) k_dual(SweepArgs a, int n_groups) {
     using E = Ent<L, LAYOUT>;
     using T = DualTile<E::M, E::W>;
     constexpr int W = E::W, NG = T::NG, Q = T::Q;
+    const int ng = PART ? n_groups : NG;
     constexpr uint32_t FULL = 0xFFFFFFFFu;
     __shared__ uint32_t s_th[T::WARPS][NG * W][32];        // staged dual words, [group, word][lane]
     __shared__ uint4 s_q[T::WARPS][Q];                     // queued tie words
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t below = (1u << lane) - 1u;
     const uint64_t n_items = (uint64_t)a.E * a.C;          // < 2^32 (checked by the host)
-    const uint64_t base = ((uint64_t)blockIdx.x * T::WARPS + warp) * (NG * 32);
+    const uint64_t base = ((uint64_t)blockIdx.x * T::WARPS + warp) * (ng * 32);
     const uint32_t sweep = (uint32_t)a.ctl->sweep;
     const uint8_t* xin = a.x + (size_t)(sweep & 1) * a.N * a.C;
     int nq = 0;                                            // entries queued (warp-uniform)
 #pragma unroll 1
-    for (int j = 0; j < NG; ++j) {
+    for (int j = 0; j < ng; ++j) {
         const uint64_t g64 = base + 32 * j + lane;
         const uint32_t g = (uint32_t)g64;
         const bool in_range = g64 < n_items;
@@ -473,7 +477,7 @@ __global__ void __launch_bounds__(256, FEW ? 2 : 4) k_dual(SweepArgs a) {
     }
     __syncwarp();
 #pragma unroll 1
-    for (int j = 0; j < NG; ++j) {
+    for (int j = 0; j < ng; ++j) {
         const uint64_t g64 = base + 32 * j + lane;
         if (g64 >= n_items) break;
         uint32_t* out = a.theta + g64 * W;
@@ -1099,6 +1103,107 @@ __global__ void __launch_bounds__(128, PrimalPipe<L, LAYOUT, CH>::BLOCKS) k_prim
         __syncwarp();                                                    // this half is free for the unit after the next
         code = code1;
         code1 = code2;
+    }
+}
+
+// Label-per-lane form for models that leave the thread form too few warps: G
+// lanes (a power of two, at least L) share a (site, chain) item and lane x sums
+// label x's field -- the entries of row x of an incidence where the site is the
+// source, of column x where it is the destination, in entry order, two-sum
+// flush every 32 incidences: the additions of k_primal into that label, bit for
+// bit.  The first lane gathers the fields and draws.  A lane has L - 1 entries of
+// an incidence instead of (L - 1)^2 and their weights are loaded side by side:
+// 25,611 sites of degree 15, L = 8, one chain: 83 -> 34 us.
+template <int L>
+struct LabelLanes {
+    static constexpr int G = L <= 8 ? 8 : 16;
+};
+
+template <int L, int LAYOUT, bool POT = false>
+__global__ void __launch_bounds__(256) k_primal_labels(SweepArgs a) {
+    using E = Ent<L, LAYOUT>;
+    constexpr int G = LabelLanes<L>::G, W = E::W, MP = E::MP;
+    constexpr int R = L - 1;                               // entries of a label per incidence
+    static_assert(W <= 2 && LAYOUT == MRF_LAYOUT_PIVOT, "full tables of at most 64 entries");
+    const uint64_t id = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const uint64_t g64 = id / G;
+    const int x = (int)(id % G);
+    const bool item = g64 < (uint64_t)a.N * a.C;
+    const uint32_t g = item ? (uint32_t)g64 : 0u;
+    const uint32_t v = a.fdC.div(g), c = g - v * (uint32_t)a.C;
+    const uint32_t sweep = (uint32_t)a.ctl->sweep;
+    const int64_t p0 = a.inc_ptr[v];
+    int64_t p1 = a.inc_ptr[v + 1];
+    const bool active = item && p1 - p0 <= a.hub_deg;             // else k_primal_hub's
+    const bool has = active && x < L && x > 0;                    // label 0 has no entries
+    if (!has) p1 = p0;
+    float acc = 0.0f, hi = 0.0f, lo = 0.0f;
+    int chunk = 0;
+    bool flushed = false;
+    constexpr int B = 4;                                   // incidences whose words and weights are loaded together
+    for (int64_t base = p0; base < p1; base += B) {
+        int code[B];
+        uint64_t bits[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) code[u] = base + u < p1 ? __ldg(&a.inc[base + u].x) : -1;
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            bits[u] = 0;
+            if (code[u] >= 0) {
+                const uint32_t* th = a.theta + ((int64_t)(code[u] >> 1) * a.C + c) * W;
+                if constexpr (W == 2) {
+                    const uint2 q = __ldg(reinterpret_cast<const uint2*>(th));
+                    bits[u] = (uint64_t)q.y << 32 | q.x;
+                } else {
+                    bits[u] = __ldg(th);
+                }
+            }
+        }
+        float t[B][R];
+        int first[B], step[B];
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const bool dst = code[u] & 1;
+            first[u] = dst ? x - 1 : (x - 1) * R;
+            step[u] = dst ? R : 1;
+            const float* tau = a.tau + (int64_t)(code[u] >= 0 ? code[u] >> 1 : 0) * MP;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const float w = __ldg(tau + first[u] + i * step[u]);
+                t[u][i] = dst ? fabsf(w) : w;
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            if (code[u] < 0) continue;
+            const uint64_t b = bits[u] >> first[u];
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+                if ((b >> (i * step[u])) & 1u) acc += t[u][i];
+            if (++chunk == 32) {
+                two_sum_add(hi, lo, acc);
+                acc = 0.0f;
+                chunk = 0;
+                flushed = true;
+            }
+        }
+    }
+    float f = 0.0f;
+    if (active && x < L) {
+        const float ut = __ldg(a.utf + (int64_t)v * L + x);
+        // (an unflushed pair is zero: hi + lo = acc exactly)
+        if (flushed) two_sum_add(hi, lo, acc);
+        f = ut + (flushed ? hi + lo : acc);
+        if (POT) a.pot[((int64_t)v * L + x) * a.C + c] = f;
+    }
+    if (POT) return;
+    float F[L];
+#pragma unroll
+    for (int y = 0; y < L; ++y) F[y] = __shfl_sync(0xffffffffu, f, y, G);
+    if (active && x == 0) {
+        uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
+        float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
+        xout[g] = (uint8_t)draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl, a.lpv ? a.lpv + g : nullptr);
     }
 }
 
@@ -1896,10 +2001,18 @@ cudaError_t run_dual(const SweepArgs& a, cudaStream_t s) {
     // few chains and wide tables (two groups per warp): 128 registers and two blocks per SM; at 64
     // registers the 8-word form spills (224 B); with one chain on 25.2 M edges of L = 16 (the
     // 2,000-graph batch's largest class) it measured 5.14 vs 4.12 ms per sweep
-    if (a.C < 32 && T::NG <= 2)
-        k_dual<L, LAYOUT, true><<<blocks_for(n, 32 * T::NG * T::WARPS), 32 * T::WARPS, 0, s>>>(a);
-    else
-        k_dual<L, LAYOUT><<<blocks_for(n, 32 * T::NG * T::WARPS), 32 * T::WARPS, 0, s>>>(a);
+    // groups per warp: NG, or as many as leave four blocks per SM (199,852 edges of L = 2, one chain,
+    // 16 groups per warp are 49 blocks: 33 us, 9 us with one)
+    const int ng = (int)std::min<int64_t>(T::NG, std::max<int64_t>(1, n / (32 * T::WARPS * 152 * 4)));
+    const unsigned blocks = blocks_for(n, 32 * ng * T::WARPS);
+    if (a.C < 32 && T::NG <= 2) {
+        if (ng < T::NG) k_dual<L, LAYOUT, (T::NG <= 2), true><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);
+        else k_dual<L, LAYOUT, (T::NG <= 2)><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);
+    } else if (ng < T::NG) {
+        k_dual<L, LAYOUT, false, true><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);
+    } else {
+        k_dual<L, LAYOUT><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);
+    }
     return cudaGetLastError();
 }
 
@@ -1964,7 +2077,21 @@ cudaError_t run_field(const SweepArgs& args, cudaStream_t s) {
     const bool hubs = a.max_deg > kHubDegree && a.max_deg != 0x7FFFFFFF;
     if (hubs) a.hub_deg = kHubDegree;
     cudaError_t e = cudaSuccess;
-    if (a.C % 32 == 0) {
+    bool labels = false;
+    if constexpr (LAYOUT == MRF_LAYOUT_PIVOT && L >= 5 && L <= 9) {
+        // Few items: a lane per label.  us per launch, thread form / label lanes, lattices of L = 8:
+        // 1,728 items 16 / 8, 13,824 18 / 11, 20,480 17 / 14, 32,768 17 / 17, 69,120 17 / 27; 25,611
+        // sites of degree 15: 83 / 34; L = 6: 8,192 items 11 / 8, 65,536 12 / 24; L = 4: no gain.  With a
+        // multiple of 32 chains the warp form is faster (16,384 items: 8 / 12).
+        labels = a.C % 32 != 0 && n <= (L >= 7 ? 32768 : 16384);
+        if (labels) {
+            k_primal_labels<L, LAYOUT, POT><<<blocks_for(n * LabelLanes<L>::G, 256), 256, 0, s>>>(a);
+            e = cudaGetLastError();
+        }
+    }
+    if (labels) {
+        // done
+    } else if (a.C % 32 == 0) {
         e = run_primal_warps<L, LAYOUT, POT>(a, s);
     } else {
         k_primal<L, LAYOUT, false, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);

@@ -56,6 +56,12 @@ def test_lattice_forms_match_the_oracle(L, C, shape):
     _check(wl.potts_grid3d(*shape, L=L, seed=40 + L), C, 1000 + L)
 
 
+@pytest.mark.parametrize("L,C,E,N", [(5, 1, 900, 200), (6, 7, 400, 150), (7, 2, 600, 40), (8, 1, 1500, 70), (9, 3, 300, 90)])
+def test_label_lanes_match_the_oracle(L, C, E, N):
+    # a lane per label: odd item counts, degrees on both sides of a two-sum flush (32)
+    _check(wl.tiny_random(N, L, E, w_std=0.3, seed=110 + L), C, 5000 + L)
+
+
 @pytest.mark.parametrize("L,C", [(4, 64), (8, 64), (8, 32), (16, 64)])
 def test_diagonal_tables_match_the_oracle(L, C):
     _check(wl.ferro_potts_grid3d(5, 4, 3, L=L, seed=50 + L), C, 2000 + L)
