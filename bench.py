@@ -260,12 +260,12 @@ def run_ours(args, ws, rank, local):
     h.sweep(k_split, mode)
     ktimes = h.kernel_times()
     h.set_kernel_timing(False)
-    # launches per sweep of the library's kernels (+ k_advance, which is not timed),
+    # launches per sweep of the library's kernels,
     # counted in the split run; the graph of a sweep replays the same launches
     if "k_sweep_small" in ktimes or "k_sw_small" in ktimes:
         launches = 1                              # a small model runs all sweeps of a call in one launch
     else:
-        per_sweep = sum(n * KERNELS_PER_RECORD.get(k, 1) for k, (_, n) in ktimes.items()) / k_split + 1
+        per_sweep = sum(n * KERNELS_PER_RECORD.get(k, 1) for k, (_, n) in ktimes.items()) / k_split
         launches = int(round(per_sweep * args.steps))
 
     # roofline of the dominant kernel (device time from the per-kernel split run)
@@ -726,7 +726,7 @@ def run_batch_workload(args):
         kt = {n: v[0] / v[1] for n, v in raw.items()}
         row = {"L": hk.L, "sites": hk.N, "edges": int(inf.n_edges), "edge_slots": int(inf.n_edge_slots),
                "dual_bits_per_edge": int(inf.n_entries), "kernels_ms": kt,
-               "launches_per_sweep": sum(v[1] for v in raw.values()) / 3 + 1,          # + k_advance (not timed)
+               "launches_per_sweep": sum(v[1] for v in raw.values()) / 3,
                "two_label_unaries": hk.L == 2}
         per_class.append(row)
         for name, ms in kt.items():
@@ -1302,7 +1302,7 @@ def run_learned_workload(args):
     h.sweep(5, M.MODE_LEARNED)
     kt_raw = h.kernel_times()
     kt_learned = {k: v[0] / v[1] for k, v in kt_raw.items()}
-    launches_per_sweep = sum(v[1] for v in kt_raw.values()) / 5 + 1          # + k_advance (not timed)
+    launches_per_sweep = sum(v[1] for v in kt_raw.values()) / 5
     h.sweep(5, M.MODE_PLAIN)
     kt_plain = {k: v[0] / v[1] for k, v in h.kernel_times().items()}
     h.set_kernel_timing(False)

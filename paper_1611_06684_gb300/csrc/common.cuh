@@ -41,7 +41,7 @@ struct Ctl {
     unsigned long long count_from;     // sweeps with t >= count_from are counted
     unsigned long long boundary;       // draws within 1e-6 of a decision boundary
     uint32_t splash_offset;            // packed (ox | oy << 8 | oz << 16) of the last blocked sweep
-    uint32_t done;                     // clusters of a small-model launch that have finished (0 between launches)
+    uint32_t done;                     // blocks or clusters of the launch that advances the index that have finished (0 between launches)
 };
 
 static_assert(sizeof(Ctl) == 32, "part of the checkpoint format");
@@ -250,7 +250,6 @@ bool mlp_tc_supported(const LearnedArgs& a);
 int64_t mlp_tc_image_bytes(int H, int O, int Kx);
 cudaError_t launch_mlp_images(const LearnedArgs& a, cudaStream_t s);
 cudaError_t launch_learned_mlp_tc(const LearnedArgs& a, cudaStream_t s);
-cudaError_t launch_advance(const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_splash(const SweepArgs& a, int layout, cudaStream_t s);
 cudaError_t launch_splash_offset(const SweepArgs& a, cudaStream_t s, int64_t iter = -1);
 cudaError_t launch_tree_map(const SweepArgs& a, uint8_t* xout, cudaStream_t s);
@@ -339,6 +338,9 @@ struct DecompArgs {
     const uint32_t* status;
 };
 cudaError_t launch_check_finite(const float* p, int64_t n, unsigned long long* bad, cudaStream_t s);
+// out[0 .. kSumBlocks): partial sums of p in a fixed order.
+constexpr int kSumBlocks = 152;
+cudaError_t launch_sum_double(const double* p, int64_t n, double* out, cudaStream_t s);
 cudaError_t launch_count_offdiag(const float* pair, int64_t n_edges, int L, unsigned long long* nz, cudaStream_t s);
 cudaError_t launch_decompose(const DecompArgs& a, cudaStream_t s);
 cudaError_t launch_build_planes(const uint32_t* thr, int64_t n, const int64_t* slots, int64_t first_slot, int M,

@@ -224,6 +224,23 @@ __global__ void k_fold_unary(const float* unary, const double* unary_d, const do
     if (utf) utf[i] = (float)acc;
 }
 
+__global__ void __launch_bounds__(256) k_sum_double(const double* __restrict__ p, int64_t n, double* __restrict__ out) {
+    __shared__ double s_sum[256];
+    double acc = 0.0;
+    for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < n; i += gridDim.x * 256ll) acc += p[i];
+    s_sum[threadIdx.x] = acc;
+    for (int o = 128; o > 0; o >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < o) s_sum[threadIdx.x] += s_sum[threadIdx.x + o];
+    }
+    if (threadIdx.x == 0) out[blockIdx.x] = s_sum[0];
+}
+
+cudaError_t launch_sum_double(const double* p, int64_t n, double* out, cudaStream_t s) {
+    k_sum_double<<<kSumBlocks, 256, 0, s>>>(p, n, out);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_check_finite(const float* p, int64_t n, unsigned long long* bad, cudaStream_t s) {
     if (n > 0) k_check_finite<<<1216, 256, 0, s>>>(p, n, bad);
     return cudaGetLastError();

@@ -12,6 +12,9 @@
 
 using namespace mrfk;
 
+// 64-bit words of a handle's flag buffer: counters of the checks, then the partial sums of the log constant.
+constexpr int kFlagWords = 8 + kSumBlocks;
+
 struct mrf {
     int32_t N = 0, L = 0, C = 0, layout = MRF_LAYOUT_PIVOT, M = 0, W = 0;
     int64_t E_live = 0, E_slots = 0, E_cap = 0;
@@ -83,7 +86,8 @@ struct mrf {
     bool sw_checked = false;           // the model passed the check since the factors last changed
     float* d_pot = nullptr;            // [N][L][C] node potentials of the blocked sweep
     float* d_part = nullptr;           // [E_cap][C][2][L] partial fields of the edge-partial plain sweep
-    int64_t part_cap = 0;              // edge slots d_part holds
+    bool tables_ok = false;            // the per-edge arrays exist, for E_cap slots of the current M, W and layout
+    int64_t resid_cap = 0;             // edges d_resid holds
     int schedule = 0;                  // primal schedule in use (1 thread, 2 CTA); 0 = not tuned yet
     int32_t* d_csr_work = nullptr;     // [2N] degrees and cursors of the device CSR build
     int64_t* d_csr_sums = nullptr;     // block sums of the device scan
@@ -447,7 +451,7 @@ mrf_status mrf_create(mrf_t** out, int32_t n_vars, int32_t n_labels, int32_t n_c
     auto bail = [&](mrf_status st) { mrf_destroy(h); return st; };
     const size_t NL = (size_t)n_vars * n_labels, NC = (size_t)n_vars * n_chains;
     if (dalloc(h->d_unary, NL) || dalloc(h->d_ut, NL) || dalloc(h->d_utf, NL) || dalloc(h->d_x, 2 * NC) || dalloc(h->d_counts, NL) ||
-        dalloc(h->d_ctl, 1) || dalloc(h->d_flag, 1)) {
+        dalloc(h->d_ctl, 1) || dalloc(h->d_flag, kFlagWords)) {
         cudaGetLastError();
         return bail(MRF_ENOMEM);
     }
@@ -499,81 +503,143 @@ mrf_status mrf_set_factors(mrf_t* h, const float* unary_log, int64_t n_edges, co
         return fail(h, MRF_EINVAL, "null pointer or negative edge count");
     if (ptr_kind != MRF_PTR_HOST && ptr_kind != MRF_PTR_DEVICE) return fail(h, MRF_EINVAL, "bad ptr_kind");
     if (n_edges >= ((int64_t)1 << 30)) return fail(h, MRF_ERANGE, "too many edges (limit 2^30)");
-    drop_graphs(h);
     const int L = h->L, N = h->N;
-    // indices: host-side checks
-    MRF_CUDA(h, to_host(h->h_src, src, n_edges, ptr_kind, h->stream));
-    MRF_CUDA(h, to_host(h->h_dst, dst, n_edges, ptr_kind, h->stream));
-    for (int64_t e = 0; e < n_edges; ++e) {
-        const int s = h->h_src[e], t = h->h_dst[e];
-        if (s < 0 || s >= N || t < 0 || t >= N) return fail(h, MRF_ERANGE, "edge " + std::to_string(e) + ": vertex id out of range");
-        if (s == t) return fail(h, MRF_ERANGE, "edge " + std::to_string(e) + ": self-loop");
-    }
-    // potentials: copy, then check on the device
-    MRF_CUDA(h, to_device(h->d_unary, unary_log, (int64_t)N * L, ptr_kind, h->stream));
-    mrf_status st = check_finite_device(h, h->d_unary, (int64_t)N * L, "unary_log");
-    if (st != MRF_OK) return st;
+    const size_t E = (size_t)n_edges;
+    cudaStream_t s = h->stream;
+    // Potentials from host memory go through a device copy; device arrays are read where they are (the
+    // call waits for the stream before it returns).  All checks are launched together and read back
+    // once: non-finite unaries, non-finite table values, off-diagonal table values.
     float* d_pair = nullptr;
-    MRF_CUDA(h, dalloc(d_pair, (size_t)n_edges * L * L));
     struct Guard { float*& p; ~Guard() { dfree(p); } } guard{d_pair};
-    MRF_CUDA(h, to_device(d_pair, pair_log, n_edges * L * L, ptr_kind, h->stream));
-    st = check_finite_device(h, d_pair, n_edges * L * L, "pair_log");
-    if (st != MRF_OK) return st;
+    const float* pair = pair_log;
+    MRF_CUDA(h, to_device(h->d_unary, unary_log, (int64_t)N * L, ptr_kind, s));
+    if (ptr_kind == MRF_PTR_HOST) {
+        MRF_CUDA(h, dalloc(d_pair, E * L * L));
+        MRF_CUDA(h, to_device(d_pair, pair_log, n_edges * L * L, ptr_kind, s));
+        pair = d_pair;
+    }
+    unsigned long long flag[3] = {0, 0, 0};
+    MRF_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(flag), s));
+    MRF_CUDA(h, launch_check_finite(h->d_unary, (int64_t)N * L, h->d_flag, s));
+    MRF_CUDA(h, launch_check_finite(pair, n_edges * L * L, h->d_flag + 1, s));
+    MRF_CUDA(h, launch_count_offdiag(pair, n_edges, L, h->d_flag + 2, s));
+    // endpoints: host mirror and host-side checks, while those kernels run
+    std::vector<int32_t> h_src, h_dst;
+    MRF_CUDA(h, to_host(h_src, src, n_edges, ptr_kind, s));
+    MRF_CUDA(h, to_host(h_dst, dst, n_edges, ptr_kind, s));
+    for (int64_t e = 0; e < n_edges; ++e) {
+        const int v = h_src[e], t = h_dst[e];
+        if (v < 0 || v >= N || t < 0 || t >= N) return fail(h, MRF_ERANGE, "edge " + std::to_string(e) + ": vertex id out of range");
+        if (v == t) return fail(h, MRF_ERANGE, "edge " + std::to_string(e) + ": self-loop");
+    }
+    MRF_CUDA(h, cudaMemcpyAsync(flag, h->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
+    MRF_CUDA(h, cudaStreamSynchronize(s));
+    if (flag[0]) return fail(h, MRF_ENONFINITE, "unary_log: " + std::to_string(flag[0]) + " non-finite values");
+    if (flag[1]) return fail(h, MRF_ENONFINITE, "pair_log: " + std::to_string(flag[1]) + " non-finite values");
     // layout: DIAG when L >= 3 and every off-diagonal entry is exactly zero
-    MRF_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(unsigned long long), h->stream));
-    MRF_CUDA(h, launch_count_offdiag(d_pair, n_edges, L, h->d_flag, h->stream));
-    unsigned long long offdiag = 0;
-    MRF_CUDA(h, cudaMemcpyAsync(&offdiag, h->d_flag, sizeof(offdiag), cudaMemcpyDeviceToHost, h->stream));
-    MRF_CUDA(h, cudaStreamSynchronize(h->stream));
-    h->layout = (L >= 3 && n_edges > 0 && offdiag == 0) ? MRF_LAYOUT_DIAG : MRF_LAYOUT_PIVOT;
+    const int layout = (L >= 3 && n_edges > 0 && flag[2] == 0) ? MRF_LAYOUT_DIAG : MRF_LAYOUT_PIVOT;
+    const bool want_resid = h->opt.grid_nx > 0 || h->opt.exact_edges;
+    // The per-edge arrays of an earlier call are kept if they fit (at most half as large again as
+    // needed): a program that sets new potentials for every frame allocates nothing.
+    const bool keep = h->tables_ok && layout == h->layout && h->E_cap >= n_edges &&
+                      h->E_cap <= n_edges + n_edges / 2 + 4096 && (!want_resid || h->resid_cap >= n_edges);
+    // A captured sweep holds the handle's pointers and sizes by value; it stays valid if none of them
+    // changes.
+    const int64_t old_edges = h->E_slots, old_inc_cap = h->inc_cap;
+    const int32_t old_deg = h->max_deg;
+    const bool had_factors = h->has_factors;
+    h->has_factors = false;                    // until every array below is in place
+    h->h_src.swap(h_src);
+    h->h_dst.swap(h_dst);
+    if (!keep) drop_graphs(h);
+    h->layout = layout;
     h->M = n_entries(L, h->layout);
     h->W = (h->M + 31) / 32;
-    h->E_live = h->E_slots = h->E_cap = n_edges;
+    h->E_live = h->E_slots = n_edges;
+    if (!keep) h->E_cap = n_edges;
     h->mirror_stale = false;
     h->free_slots.clear();
-    const bool want_resid = h->opt.grid_nx > 0 || h->opt.exact_edges;
     if (h->opt.grid_nx > 0 && !lattice_ok(h)) {
-        h->has_factors = false;
+        drop_graphs(h);
+        h->tables_ok = h->tables_ok && keep;
         return fail(h, MRF_EINVAL, "options.grid set but the edges are not the lattice's in canonical order");
     }
-    const size_t E = (size_t)n_edges;
-    MRF_CUDA(h, dalloc(h->d_src, E)); MRF_CUDA(h, dalloc(h->d_dst, E));
-    if ((uint64_t)E * h->C >= (1ull << 32)) return fail(h, MRF_ERANGE, "edges x chains must be below 2^32");
-    MRF_CUDA(h, dalloc(h->d_tau, E * pad4(h->M))); MRF_CUDA(h, dalloc(h->d_thr, E * h->M));
-    MRF_CUDA(h, dalloc(h->d_tpl, E * plane_words(h->M)));
-    MRF_CUDA(h, dalloc(h->d_fold, E * 2 * L)); MRF_CUDA(h, dalloc(h->d_cst, E));
-    if (want_resid) MRF_CUDA(h, dalloc(h->d_resid, E * L * L)); else dfree(h->d_resid);
-    if (h->layout == MRF_LAYOUT_DIAG || L == 2) {
-        MRF_CUDA(h, dalloc(h->d_swt, E * L)); MRF_CUDA(h, dalloc(h->d_swl, E * L)); MRF_CUDA(h, dalloc(h->d_swell, E * L));
-    } else {
-        dfree(h->d_swt); dfree(h->d_swl); dfree(h->d_swell);
+    if ((uint64_t)E * h->C >= (1ull << 32)) {
+        drop_graphs(h);
+        h->tables_ok = h->tables_ok && keep;
+        return fail(h, MRF_ERANGE, "edges x chains must be below 2^32");
+    }
+    if (!keep) {
+        h->tables_ok = false;
+        MRF_CUDA(h, dalloc(h->d_src, E)); MRF_CUDA(h, dalloc(h->d_dst, E));
+        MRF_CUDA(h, dalloc(h->d_tau, E * pad4(h->M))); MRF_CUDA(h, dalloc(h->d_thr, E * h->M));
+        MRF_CUDA(h, dalloc(h->d_tpl, E * plane_words(h->M)));
+        MRF_CUDA(h, dalloc(h->d_fold, E * 2 * L)); MRF_CUDA(h, dalloc(h->d_cst, E));
+        if (want_resid) MRF_CUDA(h, dalloc(h->d_resid, E * L * L)); else dfree(h->d_resid);
+        h->resid_cap = want_resid ? n_edges : 0;
+        if (h->layout == MRF_LAYOUT_DIAG || L == 2) {
+            MRF_CUDA(h, dalloc(h->d_swt, E * L)); MRF_CUDA(h, dalloc(h->d_swl, E * L)); MRF_CUDA(h, dalloc(h->d_swell, E * L));
+        } else {
+            dfree(h->d_swt); dfree(h->d_swl); dfree(h->d_swell);
+        }
+        if (L == 2) {
+            MRF_CUDA(h, dalloc(h->d_swfold, E * 2 * L)); MRF_CUDA(h, dalloc(h->d_swut, (size_t)N * L));
+        } else {
+            dfree(h->d_swfold); dfree(h->d_swut);
+        }
+        MRF_CUDA(h, dalloc(h->d_theta, E * h->C * h->W));
+        if (use_partial(h)) MRF_CUDA(h, dalloc(h->d_part, E * h->C * 2 * h->L));
+        h->tables_ok = true;
     }
     h->hg_ready = false;
-    if (L == 2) {
-        MRF_CUDA(h, dalloc(h->d_swfold, E * 2 * L)); MRF_CUDA(h, dalloc(h->d_swut, (size_t)N * L));
-    } else {
-        dfree(h->d_swfold); dfree(h->d_swut);
-    }
     h->sw_checked = false;
-    MRF_CUDA(h, dalloc(h->d_theta, E * h->C * h->W));
-    if (use_partial(h)) MRF_CUDA(h, dalloc(h->d_part, E * h->C * 2 * h->L));
-    MRF_CUDA(h, to_device(h->d_src, h->h_src.data(), n_edges, MRF_PTR_HOST, h->stream));
-    MRF_CUDA(h, to_device(h->d_dst, h->h_dst.data(), n_edges, MRF_PTR_HOST, h->stream));
-    MRF_CUDA(h, build_csr(h));
+    MRF_CUDA(h, to_device(h->d_src, src, n_edges, ptr_kind, s));
+    MRF_CUDA(h, to_device(h->d_dst, dst, n_edges, ptr_kind, s));
+    // incidence lists on the device (sites of more than 512 incidences sorted by a CTA each; on the host
+    // if one is too long for that)
+    if (!h->d_inc_ptr) MRF_CUDA(h, dalloc(h->d_inc_ptr, (size_t)N + 1));
+    if (2 * n_edges > h->inc_cap || !h->d_inc) {
+        MRF_CUDA(h, dalloc(h->d_inc, std::max<size_t>(2 * E, 1)));
+        h->inc_cap = 2 * n_edges;
+    }
+    if (!h->d_csr_work) {
+        MRF_CUDA(h, dalloc(h->d_csr_work, 2 * (size_t)N + 2));
+        MRF_CUDA(h, dalloc(h->d_csr_sums, (size_t)((N + 1 + 1023) / 1024 + 2)));
+    }
+    MRF_CUDA(h, init_csr_sort_long());
+    MRF_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(flag), s));
+    MRF_CUDA(h, build_csr_device(h->d_src, h->d_dst, n_edges, N, h->d_inc_ptr, h->d_inc, h->d_csr_work, h->d_csr_sums,
+                                 h->d_flag, 512, s));
+    MRF_CUDA(h, launch_csr_sort_long(h->d_inc_ptr, h->d_inc, N, 512, reinterpret_cast<uint32_t*>(h->d_flag + 1), s));
+    MRF_CUDA(h, launch_max_degree(h->d_inc_ptr, N, reinterpret_cast<unsigned*>(h->d_flag + 2), s));
     DecompArgs d{};
     d.L = L; d.M = h->M; d.layout = h->layout; d.n = n_edges; d.slots = nullptr; d.first_slot = 0;
-    d.pair = d_pair; d.tau = h->d_tau; d.thr = h->d_thr; d.fold = h->d_fold; d.cst = h->d_cst; d.resid = h->d_resid;
+    d.pair = pair; d.tau = h->d_tau; d.thr = h->d_thr; d.fold = h->d_fold; d.cst = h->d_cst; d.resid = h->d_resid;
     d.sw_thr = h->d_swt; d.sw_lw = h->d_swl; d.sw_fold = h->d_swfold; d.sw_ell = h->d_swell;
-    MRF_CUDA(h, launch_decompose(d, h->stream));
-    MRF_CUDA(h, launch_build_planes(h->d_thr, n_edges, nullptr, 0, h->M, h->d_tpl, h->stream));
-    MRF_CUDA(h, launch_fold_unary(h->d_unary, h->d_fold, h->d_inc_ptr, h->d_inc, N, L, h->d_ut, h->d_utf, h->stream));
-    if (h->d_swut)
-        MRF_CUDA(h, launch_fold_unary(h->d_unary, h->d_swfold, h->d_inc_ptr, h->d_inc, N, L, h->d_swut, nullptr, h->stream));
+    MRF_CUDA(h, launch_decompose(d, s));
+    MRF_CUDA(h, launch_build_planes(h->d_thr, n_edges, nullptr, 0, h->M, h->d_tpl, s));
+    auto fold = [&]() -> cudaError_t {
+        cudaError_t e = launch_fold_unary(h->d_unary, h->d_fold, h->d_inc_ptr, h->d_inc, N, L, h->d_ut, h->d_utf, s);
+        if (e == cudaSuccess && h->d_swut)
+            e = launch_fold_unary(h->d_unary, h->d_swfold, h->d_inc_ptr, h->d_inc, N, L, h->d_swut, nullptr, s);
+        return e;
+    };
+    MRF_CUDA(h, fold());
     // log constant (for log-partition estimates): sum of per-edge constants
-    std::vector<double> cst((size_t)n_edges);
-    if (n_edges) MRF_CUDA(h, cudaMemcpyAsync(cst.data(), h->d_cst, E * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    MRF_CUDA(h, cudaStreamSynchronize(h->stream));
-    h->log_const = std::accumulate(cst.begin(), cst.end(), 0.0);
+    double* d_sums = reinterpret_cast<double*>(h->d_flag + 8);
+    double sums[kSumBlocks];
+    MRF_CUDA(h, launch_sum_double(h->d_cst, n_edges, d_sums, s));
+    MRF_CUDA(h, cudaMemcpyAsync(flag, h->d_flag, sizeof(flag), cudaMemcpyDeviceToHost, s));
+    MRF_CUDA(h, cudaMemcpyAsync(sums, d_sums, sizeof(sums), cudaMemcpyDeviceToHost, s));
+    MRF_CUDA(h, cudaStreamSynchronize(s));
+    h->max_deg = (int32_t)flag[2];
+    if (flag[1]) {
+        MRF_CUDA(h, build_csr(h));
+        MRF_CUDA(h, fold());
+        MRF_CUDA(h, cudaStreamSynchronize(s));
+    }
+    if (!had_factors || n_edges != old_edges || h->max_deg != old_deg || h->inc_cap != old_inc_cap || flag[1]) drop_graphs(h);
+    h->log_const = std::accumulate(sums, sums + kSumBlocks, 0.0);
     h->has_factors = true;
     h->schedule = 0;
     return MRF_OK;
@@ -935,7 +1001,6 @@ static mrf_status enqueue_sweep(mrf_t* h, int mode) {
         if (e == cudaSuccess) e = timed(h, MRF_K_FFBS, [&] { return launch_ffbs(a, s); });
     }
     if (e == cudaSuccess) e = timed(h, MRF_K_ACCUMULATE, [&] { return launch_accumulate(a, s); });
-    if (e == cudaSuccess) e = launch_advance(a, s);
     if (e != cudaSuccess) { cudaGetLastError(); return fail(h, MRF_ECUDA, std::string("sweep launch: ") + cudaGetErrorString(e)); }
     return MRF_OK;
 }

@@ -22,11 +22,9 @@ __global__ void k_init_labels(SweepArgs a) {
 // counts[v][a] += #{c : x_new[v][c] = a} for counted sweeps.  Per-label
 // counts of up to 255 chains per pass are kept as sixteen 8-bit lanes of two
 // 64-bit registers (label x adds 1 << 8x to the low or high word).
-__global__ void k_accumulate(SweepArgs a) {
-    const int v = blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= a.N) return;
-    const unsigned long long t = a.ctl->sweep;
-    if (t < a.ctl->count_from) return;
+// The last block to finish advances the sweep index (a launch of its own took
+// 2.5 us per sweep).
+__device__ __forceinline__ void count_labels(const SweepArgs& a, int v, unsigned long long t) {
     const uint8_t* xo = a.x + (size_t)((t + 1) & 1) * a.N * a.C + (int64_t)v * a.C;
     uint32_t tot[kMaxLabels];
 #pragma unroll
@@ -63,7 +61,19 @@ __global__ void k_accumulate(SweepArgs a) {
         if (x < a.L && tot[x]) cnt[x] += tot[x];
 }
 
-__global__ void k_advance(Ctl* ctl) { ctl->sweep += 1; }
+__global__ void __launch_bounds__(256) k_accumulate(SweepArgs a) {
+    const unsigned long long t = a.ctl->sweep;
+    const int v = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= a.ctl->count_from && v < a.N) count_labels(a, v, t);
+    __syncthreads();                                       // every thread of the block has read the index
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&a.ctl->done, 1u) + 1u == gridDim.x) {
+            a.ctl->done = 0u;
+            a.ctl->sweep = t + 1;
+        }
+    }
+}
 
 // Label layout conversion between the internal x[v][c] (chain-innermost) and
 // the ABI view y[c][v], through 32x32 shared-memory tiles.
@@ -337,11 +347,6 @@ cudaError_t launch_fused(const SweepArgs& a, int layout, int schedule, cudaStrea
 
 cudaError_t launch_accumulate(const SweepArgs& a, cudaStream_t s) {
     k_accumulate<<<(a.N + 255) / 256, 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_advance(const SweepArgs& a, cudaStream_t s) {
-    k_advance<<<1, 1, 0, s>>>(a.ctl);
     return cudaGetLastError();
 }
 

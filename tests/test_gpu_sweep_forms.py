@@ -152,3 +152,71 @@ def test_hub_potentials_do_not_depend_on_the_chain_count(C):
         for _ in range(3):
             h.sweep(1, M.MODE_HIGDON)
     assert np.array_equal(many.get_labels()[:3], few.get_labels())
+
+
+def _set(h, m, device):
+    import torch
+    arrays = (m.unary, m.src, m.dst, m.pair)
+    if device:
+        arrays = tuple(torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in arrays)
+        torch.cuda.synchronize()
+    h.set_factors(*arrays)
+
+
+@pytest.mark.parametrize("device", [False, True])
+def test_set_factors_again_equals_a_new_handle(device):
+    """New potentials, then models of other edges, degrees, sizes and layouts on one handle (its arrays
+    and captured sweeps are kept where they fit), and a refused model in between."""
+    import torch
+    N, L, C = 360, 4, 6
+    models = [wl.potts_grid3d(10, 9, 4, L=L, seed=1), wl.potts_grid3d(10, 9, 4, L=L, seed=2),
+              wl.tiny_random(N, L, 900, w_std=0.4, seed=3), wl.tiny_random(N, L, 700, w_std=0.4, seed=4),
+              wl.ferro_potts_graph(N, L, 800, seed=5), wl.tiny_random(N, L, 5000, w_std=0.2, seed=6),
+              wl.Model(N, L, np.zeros((N, L), np.float32), np.zeros(0, np.int32), np.zeros(0, np.int32),
+                       np.zeros((0, L, L), np.float32)),
+              wl.potts_grid3d(10, 9, 4, L=L, seed=7)]
+    bad = wl.tiny_random(N, L, 50, seed=8)
+    bad.dst[7] = N
+    stream = torch.cuda.Stream()
+    h = M.MRF(N, L, C, seed=9, stream=stream.cuda_stream, schedule=1)
+    for i, m in enumerate(models):
+        _set(h, m, device)
+        if i == 3:
+            with pytest.raises(M.MrfError) as err:
+                _set(h, bad, device)
+            assert err.value.status == M.MRF_ERANGE and "edge 7" in str(err.value)
+            bad.dst[7] = 0 if bad.src[7] else 1
+            bad.pair[3, 1, 1] = np.inf
+            with pytest.raises(M.MrfError) as err:
+                _set(h, bad, device)
+            assert err.value.status == M.MRF_ENONFINITE
+            _set(h, m, device)
+        fresh = M.MRF(N, L, C, seed=9, stream=stream.cuda_stream, schedule=1)
+        _set(fresh, m, False)
+        fresh.set_labels(h.get_labels())
+        fresh.set_sweep_index(h.info().sweep_index)
+        for g in (h, fresh):
+            g.reset_marginals(0)
+            g.sweep(1)
+            g.sweep(3)
+        assert np.array_equal(h.get_labels(), fresh.get_labels())
+        assert np.array_equal(h.counts(), fresh.counts())
+        for x, y in zip(h.debug_tables(), fresh.debug_tables()):
+            assert np.array_equal(x, y)
+        assert abs(h.info().log_const - fresh.info().log_const) <= 1e-9 * max(1.0, abs(fresh.info().log_const))
+        if i == 2:                                         # edits after a second model
+            for g in (h, fresh):
+                g.edit_factors(np.array([5, 6]), np.array([1], np.int32), np.array([300], np.int32),
+                               np.full((1, L, L), 0.1, np.float32))
+                g.sweep(2)
+            assert np.array_equal(h.get_labels(), fresh.get_labels())
+        fresh.close()
+
+
+def test_set_factors_sorts_long_incidence_lists():
+    # a site of 3,000 incidences (the CTA sort) beside short lists, against the oracle
+    rng = np.random.default_rng(0)
+    n = 3001
+    m = wl.Model(n, 3, rng.normal(size=(n, 3)).astype(np.float32), np.zeros(n - 1, np.int32), np.arange(1, n, dtype=np.int32),
+                 rng.normal(0, 0.1, (n - 1, 3, 3)).astype(np.float32))
+    _check(m, 3, 6000)
