@@ -609,6 +609,43 @@ __device__ __forceinline__ void add_side_chains(const uint32_t (&bits)[CH][Ent<L
     else add_rows<L, LAYOUT, GLOBAL, CH, 0>(bits, t4, tv, 1, acc);
 }
 
+// The same with a test and an add per entry: for the thread form (k_primal) of 13
+// to 15 labels, whose sums spill at 64 registers either way (36,000 sites, 18
+// chains: L = 14 145 us against 159, L = 15 163 against 183; L = 12 and below
+// even, L = 16 238 against 210).
+template <int L, int LAYOUT>
+constexpr bool kSingleAdds = LAYOUT == MRF_LAYOUT_PIVOT && L >= 13 && L <= 15;
+
+template <int L, int LAYOUT>
+__device__ __forceinline__ void add_side_single(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
+                                                int side, float (&acc)[L]) {
+    using E = Ent<L, LAYOUT>;
+    const float4* t4 = reinterpret_cast<const float4*>(tau_e);
+    if (side == 0) {
+#pragma unroll
+        for (int k4 = 0; k4 < E::MP / 4; ++k4) {
+            const float4 q = __ldg(t4 + k4);
+            const float tv[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = 4 * k4 + u;
+                if (k < E::M && ((bits[k >> 5] >> (k & 31)) & 1u)) acc[E::i(k)] += tv[u];
+            }
+        }
+    } else {
+#pragma unroll
+        for (int k4 = 0; k4 < E::MP / 4; ++k4) {
+            const float4 q = __ldg(t4 + k4);
+            const float tv[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = 4 * k4 + u;
+                if (k < E::M && ((bits[k >> 5] >> (k & 31)) & 1u)) acc[E::j(k)] += fabsf(tv[u]);
+            }
+        }
+    }
+}
+
 template <int L, int LAYOUT, bool GLOBAL = true>
 __device__ __forceinline__ void add_side(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
                                          int side, float (&acc)[L]) {
@@ -688,7 +725,8 @@ __global__ void __launch_bounds__(256, FUSED ? 2 : 4) k_primal(SweepArgs a) {
 #pragma unroll
         for (int u = 0; u < B; ++u) {
             if (ic[u].x < 0) continue;
-            add_side<L, LAYOUT>(bits[u], a.tau + (ic[u].x >> 1) * (int64_t)E::MP, ic[u].x & 1, acc);
+            if constexpr (kSingleAdds<L, LAYOUT>) add_side_single<L, LAYOUT>(bits[u], a.tau + (ic[u].x >> 1) * (int64_t)E::MP, ic[u].x & 1, acc);
+            else add_side<L, LAYOUT>(bits[u], a.tau + (ic[u].x >> 1) * (int64_t)E::MP, ic[u].x & 1, acc);
             if (++chunk == 32) {
 #pragma unroll
                 for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], acc[x]); acc[x] = 0.0f; }
@@ -712,6 +750,60 @@ __global__ void __launch_bounds__(256, FUSED ? 2 : 4) k_primal(SweepArgs a) {
         for (int x = 0; x < L; ++x) pv[(int64_t)x * a.C] = F[x];
         return;
     }
+    float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
+    xout[g] = (uint8_t)draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl, a.lpv ? a.lpv + g : nullptr);
+}
+
+// Thread form for sites of at most KB incidences: every incidence code, then
+// every dual word of the site is loaded before any is used (two dependent loads
+// where batches of four made four), and no two-sum pair is kept, since no sum
+// reaches 32 incidences.  Keeps k_primal's order of additions.  151,951 sites of a
+// lattice, L = 5, 24 chains: 120 -> 101 us.
+template <int L, int LAYOUT, bool POT = false>
+__global__ void __launch_bounds__(256, 4) k_primal_low(SweepArgs a) {
+    using E = Ent<L, LAYOUT>;
+    constexpr int W = E::W, KB = 8;
+    static_assert(W <= 2, "the dual words of KB incidences are in registers");
+    const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;     // N * C < 2^32 (checked by the host)
+    if (g >= (uint64_t)a.N * a.C) return;
+    const uint32_t v = a.fdC.div(g), c = g - v * (uint32_t)a.C;
+    const int64_t p0 = a.inc_ptr[v];
+    const int deg = (int)(a.inc_ptr[v + 1] - p0);
+    int code[KB];
+#pragma unroll
+    for (int u = 0; u < KB; ++u) code[u] = u < deg ? __ldg(&a.inc[p0 + u].x) : -1;
+    uint32_t bits[KB][W];
+#pragma unroll
+    for (int u = 0; u < KB; ++u) {
+        if (code[u] < 0) continue;
+        const uint32_t* th = a.theta + ((uint64_t)((uint32_t)code[u] >> 1) * (uint32_t)a.C + c) * W;
+        if constexpr (W == 2) {
+            const uint2 q = __ldcs(reinterpret_cast<const uint2*>(th));
+            bits[u][0] = q.x;
+            bits[u][1] = q.y;
+        } else {
+            bits[u][0] = __ldcs(th);
+        }
+    }
+    float acc[L];
+#pragma unroll
+    for (int x = 0; x < L; ++x) acc[x] = 0.0f;
+#pragma unroll
+    for (int u = 0; u < KB; ++u)
+        if (code[u] >= 0)
+            add_side<L, LAYOUT>(bits[u], a.tau + (uint64_t)((uint32_t)code[u] >> 1) * E::MP, code[u] & 1, acc);
+    float F[L];
+    const float* uf = a.utf + (int64_t)v * L;
+#pragma unroll
+    for (int x = 0; x < L; ++x) F[x] = __ldg(uf + x) + acc[x];
+    if (POT) {
+        float* pv = a.pot + (int64_t)v * L * a.C + c;
+#pragma unroll
+        for (int x = 0; x < L; ++x) pv[(int64_t)x * a.C] = F[x];
+        return;
+    }
+    const uint32_t sweep = (uint32_t)a.ctl->sweep;
+    uint8_t* xout = a.x + (size_t)((sweep + 1) & 1) * a.N * a.C;
     float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
     xout[g] = (uint8_t)draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl, a.lpv ? a.lpv + g : nullptr);
 }
@@ -1530,19 +1622,20 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() { cluster_arrive(); cluster_wait(); }
 
-// Dual words of one (edge, chain) and one incidence side, from L2.
-template <int W>
-__device__ __forceinline__ void load_words_cg(const uint32_t* th, uint32_t (&bits)[W]) {
+// Dual words of one (edge, chain), written by another CTA of the cluster (L2) or by this one.
+template <int W, bool L2>
+__device__ __forceinline__ void load_words(const uint32_t* th, uint32_t (&bits)[W]) {
     if constexpr (W % 2 == 0) {
 #pragma unroll
         for (int w = 0; w < W; w += 2) {
-            const uint2 q = __ldcg(reinterpret_cast<const uint2*>(th + w));
+            const uint2* p = reinterpret_cast<const uint2*>(th + w);
+            const uint2 q = L2 ? __ldcg(p) : *p;
             bits[w] = q.x;
             bits[w + 1] = q.y;
         }
     } else {
 #pragma unroll
-        for (int w = 0; w < W; ++w) bits[w] = __ldcg(th + w);
+        for (int w = 0; w < W; ++w) bits[w] = L2 ? __ldcg(th + w) : th[w];
     }
 }
 
@@ -1557,13 +1650,19 @@ __device__ __forceinline__ void load_words_cg(const uint32_t* th, uint32_t (&bit
 // memory by every thread and advanced by the last cluster to finish.
 // Bound by latency (two barriers and their dependent L2 round trips).  50 x 50
 // Ising grid, 10 chains, 10 sweeps: 990 us in one CTA with all chains, 62 us here.
-template <int L, int LAYOUT>
+// CLUSTER = false: one CTA per group of chains, labels and dual words through
+// its L1 (no barrier's acquire drops the lines of its tables either).
+template <int L, int LAYOUT, bool CLUSTER>
 __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, FastDiv fdn) {
     using E = Ent<L, LAYOUT>;
     constexpr int W = E::W;
-    uint32_t rank, size;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(size));
+    uint32_t rank = 0, size = 1;
+    if (CLUSTER) {
+        asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(size));
+    }
+    auto label = [](const uint8_t* p) -> int { return CLUSTER ? __ldcg(p) : *p; };
+    auto barrier = [] { if (CLUSTER) cluster_barrier(); else __syncthreads(); };
     const uint32_t nc = fdn.d, cluster = blockIdx.x / size;
     const uint32_t c0 = cluster * nc;
     const uint32_t tid = rank * blockDim.x + threadIdx.x, T = size * blockDim.x;
@@ -1580,7 +1679,7 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
             const int s = a.src[e];
             if (s >= 0) {
                 const int t = a.dst[e];
-                dual_bits<L, LAYOUT>(e, c, __ldcg(xin + (int64_t)s * C + c), __ldcg(xin + (int64_t)t * C + c),
+                dual_bits<L, LAYOUT>(e, c, label(xin + (int64_t)s * C + c), label(xin + (int64_t)t * C + c),
                                      a.tpl + (int64_t)e * E::PW, a.thr + (int64_t)e * E::M, sweep, a.rk, bits);
             } else {
 #pragma unroll
@@ -1588,10 +1687,9 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
             }
             uint32_t* out = a.theta + ((int64_t)e * C + c) * W;
 #pragma unroll
-            for (int w = 0; w < W; ++w) __stcg(out + w, bits[w]);
+            for (int w = 0; w < W; ++w) out[w] = bits[w];
         }
-        if (size > 1) cluster_barrier();
-        else __syncthreads();
+        barrier();
         for (uint32_t i = tid; i < nv; i += T) {
             const uint32_t v = fdn.div(i), c = c0 + (i - v * nc);
             if (c >= C) continue;
@@ -1609,7 +1707,7 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
                 for (int u = 0; u < B; ++u) code[u] = base + u < p1 ? __ldg(&a.inc[base + u].x) : -1;
 #pragma unroll
                 for (int u = 0; u < B; ++u)
-                    if (code[u] >= 0) load_words_cg<W>(a.theta + ((int64_t)(code[u] >> 1) * C + c) * W, bits[u]);
+                    if (code[u] >= 0) load_words<W, CLUSTER>(a.theta + ((int64_t)(code[u] >> 1) * C + c) * W, bits[u]);
 #pragma unroll
                 for (int u = 0; u < B; ++u) {
                     if (code[u] < 0) continue;
@@ -1633,11 +1731,10 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
             }
             float* lp = a.logp ? a.logp + ((int64_t)c * a.N + v) * L : nullptr;
             const int lab = draw_label<L>(F, v, c, sweep, a.rk, PH_PRIMAL, lp, a.ctl);
-            __stcg(xout + (int64_t)v * C + c, (uint8_t)lab);
+            xout[(int64_t)v * C + c] = (uint8_t)lab;
             if (sweep >= count_from) atomicAdd(a.counts + (int64_t)v * L + lab, 1u);
         }
-        if (size > 1) cluster_barrier();
-        else __syncthreads();
+        barrier();
     }
     // after the last barrier every thread of the cluster has read the index
     if (rank == 0 && threadIdx.x == 0) {
@@ -2003,7 +2100,9 @@ cudaError_t run_dual(const SweepArgs& a, cudaStream_t s) {
     // 2,000-graph batch's largest class) it measured 5.14 vs 4.12 ms per sweep
     // groups per warp: NG, or as many as leave four blocks per SM (199,852 edges of L = 2, one chain,
     // 16 groups per warp are 49 blocks: 33 us, 9 us with one)
-    const int ng = (int)std::min<int64_t>(T::NG, std::max<int64_t>(1, n / (32 * T::WARPS * 152 * 4)));
+    // (wide tables: one block per SM; 102,060 items of L = 14 in two groups per warp 24 us, in one 27 us)
+    const int64_t per_sm = Ent<L, LAYOUT>::W >= 4 ? 1 : 4;
+    const int ng = (int)std::min<int64_t>(T::NG, std::max<int64_t>(1, n / (32 * T::WARPS * 152 * per_sm)));
     const unsigned blocks = blocks_for(n, 32 * ng * T::WARPS);
     if (a.C < 32 && T::NG <= 2) {
         if (ng < T::NG) k_dual<L, LAYOUT, (T::NG <= 2), true><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);
@@ -2094,7 +2193,12 @@ cudaError_t run_field(const SweepArgs& args, cudaStream_t s) {
     } else if (a.C % 32 == 0) {
         e = run_primal_warps<L, LAYOUT, POT>(a, s);
     } else {
-        k_primal<L, LAYOUT, false, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
+        bool low = false;
+        if constexpr (Ent<L, LAYOUT>::W <= 2) {
+            low = a.max_deg <= 8;
+            if (low) k_primal_low<L, LAYOUT, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
+        }
+        if (!low) k_primal<L, LAYOUT, false, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess || !hubs) return e;
@@ -2142,10 +2246,15 @@ cudaError_t run_sweep_small(const SweepArgs& a, int n_sweeps, cudaStream_t s) {
     while (size < 8 && items > 256ll * size) size *= 2;
     int64_t threads = ((items + size - 1) / size + 31) / 32 * 32;
     int64_t smem = threads <= 640 ? S::smem(a.N * nc, a.E * nc, (int)threads) : 0;
-    const bool resident = threads <= 640 && smem <= 200 * 1024;
+    // Sites of many incidences with full tables read most weights from memory in every sweep: one CTA
+    // per group of chains, whose L1 keeps them (complete graphs, 2 chains, us per 10 sweeps, cluster /
+    // one CTA: L = 6, 55 sites 639 / 464, 100 sites 1,113 / 948, 200 sites 1,945 / 2,096; L = 3, 55 sites
+    // 190 / 126; L = 2, 100 sites, 10 chains 335 / 442).
+    const bool one = a.M >= 4 && 2 * a.E >= 24 * (int64_t)a.N && items <= 5120;
+    const bool resident = threads <= 640 && smem <= 200 * 1024 && !one;
     if (!resident) {
         size = 1;
-        while (size < 8 && items > 512ll * size) size *= 2;
+        while (!one && size < 8 && items > 512ll * size) size *= 2;
         threads = 512;
         smem = 0;
     }
@@ -2161,7 +2270,9 @@ cudaError_t run_sweep_small(const SweepArgs& a, int n_sweeps, cudaStream_t s) {
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = size > 1 ? 1 : 0;
-    if (!resident) return cudaLaunchKernelEx(&cfg, k_sweep_small<L, LAYOUT>, a, n_sweeps, FastDiv::make((uint32_t)nc));
+    if (!resident)
+        return size > 1 ? cudaLaunchKernelEx(&cfg, k_sweep_small<L, LAYOUT, true>, a, n_sweeps, FastDiv::make((uint32_t)nc))
+                        : cudaLaunchKernelEx(&cfg, k_sweep_small<L, LAYOUT, false>, a, n_sweeps, FastDiv::make((uint32_t)nc));
     if (smem > 48 * 1024) {
         const cudaError_t e = cudaFuncSetAttribute(k_sweep_resident<L, LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
