@@ -2101,8 +2101,11 @@ cudaError_t run_dual(const SweepArgs& a, cudaStream_t s) {
     // groups per warp: NG, or as many as leave four blocks per SM (199,852 edges of L = 2, one chain,
     // 16 groups per warp are 49 blocks: 33 us, 9 us with one)
     // (wide tables: one block per SM; 102,060 items of L = 14 in two groups per warp 24 us, in one 27 us)
+    // The variable bound costs up to 9 %, so NG stays where it leaves two blocks per SM.
     const int64_t per_sm = Ent<L, LAYOUT>::W >= 4 ? 1 : 4;
-    const int ng = (int)std::min<int64_t>(T::NG, std::max<int64_t>(1, n / (32 * T::WARPS * 152 * per_sm)));
+    const int ng = n >= 32ll * T::WARPS * T::NG * 152 * 2
+                       ? T::NG
+                       : (int)std::min<int64_t>(T::NG, std::max<int64_t>(1, n / (32 * T::WARPS * 152 * per_sm)));
     const unsigned blocks = blocks_for(n, 32 * ng * T::WARPS);
     if (a.C < 32 && T::NG <= 2) {
         if (ng < T::NG) k_dual<L, LAYOUT, (T::NG <= 2), true><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);
