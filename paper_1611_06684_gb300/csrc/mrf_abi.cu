@@ -638,7 +638,10 @@ mrf_status mrf_set_factors(mrf_t* h, const float* unary_log, int64_t n_edges, co
         MRF_CUDA(h, fold());
         MRF_CUDA(h, cudaStreamSynchronize(s));
     }
-    if (!had_factors || n_edges != old_edges || h->max_deg != old_deg || h->inc_cap != old_inc_cap || flag[1]) drop_graphs(h);
+    // (an automatic primal schedule is chosen again on the next sweep)
+    const bool fixed_schedule = h->opt.schedule == 1 || h->opt.schedule == 2;
+    if (!had_factors || !fixed_schedule || n_edges != old_edges || h->max_deg != old_deg || h->inc_cap != old_inc_cap || flag[1])
+        drop_graphs(h);
     h->log_const = std::accumulate(sums, sums + kSumBlocks, 0.0);
     h->has_factors = true;
     h->schedule = 0;
@@ -1051,7 +1054,7 @@ mrf_status mrf_sweep(mrf_t* h, int32_t n_sweeps, int32_t mode) {
         mrf_status st = tune_schedule(h);
         if (st != MRF_OK) return st;
     }
-    // small models: all the sweeps in one single-CTA launch (launch latency dominates there)
+    // small models: all the sweeps in one launch (launch latency dominates there)
     if (mode == MRF_MODE_PLAIN && n_sweeps >= 2 && small_model(h)) {
         const SweepArgs a = make_args(h);
         MRF_CUDA(h, timed(h, MRF_K_SMALL, [&] { return launch_sweep_small(a, h->layout, n_sweeps, h->stream); }));
