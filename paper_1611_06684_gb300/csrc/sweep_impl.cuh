@@ -294,7 +294,12 @@ __device__ __forceinline__ float ex2_approx(float x) {
 // exact one; so if every |c_a - u s| is at least 2^-16 s, both give the same
 // label, and no boundary is within the 1e-6 that draw_label counts.  Takes 7
 // instructions per label where the full computation takes 18; about one draw in
-// 4,000 (L = 8) falls back to it.  NaN and infinite fields always do.
+// 4,000 (L = 8) falls back to it.
+// The rounding error of mb scales all the sums alike by 2^r, |r| up to half an
+// ulp of mb: s is in [1, L] but for that.  From fields of 1.5e9 on it can pass the
+// exponent range, where every term is 0 or infinite and the closeness test holds
+// for any label, so sums outside [2^-32, 2^32] (fields of 5e8 and more, NaN and
+// infinite fields) take the full computation.
 template <int L>
 __device__ __forceinline__ int draw_label_fast(const float (&F)[L], float u) {
     constexpr float kLog2e = 1.4426950408889634f;
@@ -317,7 +322,7 @@ __device__ __forceinline__ int draw_label_fast(const float (&F)[L], float u) {
         closest = fminf(closest, fabsf(d));
         lab += d <= 0.0f ? 1 : 0;
     }
-    return closest >= s * 0x1p-16f ? lab : -1;
+    return s >= 0x1p-32f && s <= 0x1p32f && closest >= s * 0x1p-16f ? lab : -1;
 }
 
 // Draw x_v from exp(F)/Z by the inverse CDF with the 23-bit uniform u (exact in
