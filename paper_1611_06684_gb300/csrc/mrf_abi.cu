@@ -460,6 +460,7 @@ mrf_status mrf_create(mrf_t** out, int32_t n_vars, int32_t n_labels, int32_t n_c
     if (cudaMemcpyAsync(h->d_ctl, &c0, sizeof(c0), cudaMemcpyHostToDevice, h->stream) ||
         cudaMemsetAsync(h->d_unary, 0, NL * sizeof(float), h->stream) ||
         cudaMemsetAsync(h->d_ut, 0, NL * sizeof(double), h->stream) ||
+        cudaMemsetAsync(h->d_x, 0, 2 * NC, h->stream) ||      // both halves are part of a checkpoint, written or not
         cudaMemsetAsync(h->d_counts, 0, NL * sizeof(uint32_t), h->stream)) {
         cudaGetLastError();
         return bail(MRF_ECUDA);

@@ -1922,7 +1922,11 @@ __global__ void __launch_bounds__(640) k_sweep_resident(SweepArgs a, int n_sweep
         if (has_site && sweep >= count_from) atomicAdd(a.counts + (int64_t)v * L + lab, 1u);
         wait();
     }
-    if (has_site) a.x[(size_t)(sweep & 1) * a.N * a.C + (int64_t)v * C + vc] = (uint8_t)lab;
+    if (has_site) {                                        // the last labels and, in the other half, those before
+        const int64_t g = (int64_t)v * C + vc;
+        a.x[(size_t)(sweep & 1) * a.N * a.C + g] = (uint8_t)lab;
+        a.x[(size_t)((sweep + 1) & 1) * a.N * a.C + g] = s_lab[((sweep + 1) & 1) * lab_bytes + i];
+    }
     if (rank == 0 && threadIdx.x == 0) {                   // see k_sweep_small
         __threadfence();
         if (atomicAdd(&a.ctl->done, 1u) + 1u == gridDim.x / size) {
