@@ -507,21 +507,24 @@ mrf_status mrf_set_factors(mrf_t* h, const float* unary_log, int64_t n_edges, co
     const int L = h->L, N = h->N;
     const size_t E = (size_t)n_edges;
     cudaStream_t s = h->stream;
-    // Potentials from host memory go through a device copy; device arrays are read where they are (the
-    // call waits for the stream before it returns).  All checks are launched together and read back
-    // once: non-finite unaries, non-finite table values, off-diagonal table values.
-    float* d_pair = nullptr;
-    struct Guard { float*& p; ~Guard() { dfree(p); } } guard{d_pair};
-    const float* pair = pair_log;
-    MRF_CUDA(h, to_device(h->d_unary, unary_log, (int64_t)N * L, ptr_kind, s));
+    // Potentials from host memory go through a device copy (tables, then unaries); device arrays are read
+    // where they are (the call waits for the stream before it returns).  All checks are launched together
+    // and read back once: non-finite unaries, non-finite table values, off-diagonal table values.  A call
+    // that these or the endpoint checks refuse leaves the handle's model as it was: its own unaries are
+    // written after them.
+    float* d_host = nullptr;
+    struct Guard { float*& p; ~Guard() { dfree(p); } } guard{d_host};
+    const float *pair = pair_log, *unary = unary_log;
     if (ptr_kind == MRF_PTR_HOST) {
-        MRF_CUDA(h, dalloc(d_pair, E * L * L));
-        MRF_CUDA(h, to_device(d_pair, pair_log, n_edges * L * L, ptr_kind, s));
-        pair = d_pair;
+        MRF_CUDA(h, dalloc(d_host, (E * L + N) * L));
+        MRF_CUDA(h, to_device(d_host, pair_log, n_edges * L * L, ptr_kind, s));
+        MRF_CUDA(h, to_device(d_host + E * L * L, unary_log, (int64_t)N * L, ptr_kind, s));
+        pair = d_host;
+        unary = d_host + E * L * L;
     }
     unsigned long long flag[3] = {0, 0, 0};
     MRF_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(flag), s));
-    MRF_CUDA(h, launch_check_finite(h->d_unary, (int64_t)N * L, h->d_flag, s));
+    MRF_CUDA(h, launch_check_finite(unary, (int64_t)N * L, h->d_flag, s));
     MRF_CUDA(h, launch_check_finite(pair, n_edges * L * L, h->d_flag + 1, s));
     MRF_CUDA(h, launch_count_offdiag(pair, n_edges, L, h->d_flag + 2, s));
     // endpoints: host mirror and host-side checks, while those kernels run
@@ -594,6 +597,7 @@ mrf_status mrf_set_factors(mrf_t* h, const float* unary_log, int64_t n_edges, co
     }
     h->hg_ready = false;
     h->sw_checked = false;
+    MRF_CUDA(h, to_device(h->d_unary, unary, (int64_t)N * L, MRF_PTR_DEVICE, s));
     MRF_CUDA(h, to_device(h->d_src, src, n_edges, ptr_kind, s));
     MRF_CUDA(h, to_device(h->d_dst, dst, n_edges, ptr_kind, s));
     // incidence lists on the device (sites of more than 512 incidences sorted by a CTA each; on the host
