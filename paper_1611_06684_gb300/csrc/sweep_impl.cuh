@@ -1814,7 +1814,7 @@ __global__ void __launch_bounds__(640) k_sweep_resident(SweepArgs a, int n_sweep
     }
     // edge item
     const uint32_t e = fdn.div(i), ec = c0 + (i - e * nc);
-    const bool has_edge = i < ne && ec < C && a.src[i < ne ? e : 0] >= 0;
+    const bool edge_item = i < ne && ec < C, has_edge = edge_item && a.src[e] >= 0;
     uint32_t ls = 0, lt = 0, th_s = 0, th_t = 0;           // label places of the endpoints, dual words in their owners' copies
     if (has_edge) {
         ls = (uint32_t)a.src[e] * nc + (ec - c0);
@@ -1860,6 +1860,13 @@ __global__ void __launch_bounds__(640) k_sweep_resident(SweepArgs a, int n_sweep
                 asm volatile("st.shared::cluster.u32 [%0],%1;" ::"r"(th_s + 4 * w), "r"(bits[w]) : "memory");
                 if (th_t != th_s) asm volatile("st.shared::cluster.u32 [%0],%1;" ::"r"(th_t + 4 * w), "r"(bits[w]) : "memory");
             }
+            if (it + 1 == n_sweeps) {                      // the last sweep's words are kept (mrf_debug_theta)
+#pragma unroll
+                for (int w = 0; w < W; ++w) a.theta[((int64_t)e * C + ec) * W + w] = bits[w];
+            }
+        } else if (edge_item && it + 1 == n_sweeps) {      // a free slot has none
+#pragma unroll
+            for (int w = 0; w < W; ++w) a.theta[((int64_t)e * C + ec) * W + w] = 0u;
         }
         // the random words of the next half-step are drawn while the barrier completes
         arrive();
