@@ -2199,9 +2199,15 @@ cudaError_t run_field(const SweepArgs& args, cudaStream_t s) {
     if constexpr (LAYOUT == MRF_LAYOUT_PIVOT && L >= 5 && L <= 9) {
         // Few items: a lane per label.  us per launch, thread form / label lanes, lattices of L = 8:
         // 1,728 items 16 / 8, 13,824 18 / 11, 20,480 17 / 14, 32,768 17 / 17, 69,120 17 / 27; 25,611
-        // sites of degree 15: 83 / 34; L = 6: 8,192 items 11 / 8, 65,536 12 / 24; L = 4: no gain.  With a
-        // multiple of 32 chains the warp form is faster (16,384 items: 8 / 12).
-        labels = a.C % 32 != 0 && n <= (L >= 7 ? 32768 : 16384);
+        // sites of degree 15: 83 / 34; L = 4: no gain.  With a multiple of 32 chains the warp form is
+        // faster (16,384 items: 8 / 12).  The limits are where the two meet on lattices (degree 4 to 6):
+        // the thread form gains with the chains, whose lanes share a table row, and L = 9 pays for the
+        // seven idle lanes of its sixteen (lane form over thread form, 1 / 5 / 16 chains: L = 5 at
+        // 16,000 items 1.0 / 1.06 / 1.13; L = 7 at 32,000 0.95 / 0.97 / 1.15; L = 9 at 16,000
+        // 0.81 / 1.03 / 1.14, at 32,000 1.3 / 1.7 / 1.9).
+        constexpr int few = L == 9 ? 20480 : (L >= 7 ? 32768 : 16384);
+        constexpr int many = L == 9 ? 13312 : (L == 8 ? 32768 : (L == 7 ? 24576 : (L == 6 ? 16384 : 12288)));
+        labels = a.C % 32 != 0 && n <= (a.C < 4 ? few : many);
         if (labels) {
             k_primal_labels<L, LAYOUT, POT><<<blocks_for(n * LabelLanes<L>::G, 256), 256, 0, s>>>(a);
             e = cudaGetLastError();

@@ -1,0 +1,36 @@
+"""A chain's labels do not depend on the kernel form that the number of chains
+selects: its draws depend on its own index only, and every form adds in the
+same order."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+from paper_1611_06684_gb300 import workloads as wl
+from tests.gpu_helpers import make_handle
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _gpu():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1611_06684_gb300 import build
+    build.build()
+    torch.cuda.set_device(0)
+
+
+def _same_first_chains(model, few, many, seed=5, sweeps=3):
+    a, b = make_handle(model, few, seed, use_graphs=False, schedule=1), make_handle(model, many, seed, use_graphs=False, schedule=1)
+    for _ in range(sweeps):
+        a.sweep(1)
+        b.sweep(1)
+    assert np.array_equal(a.get_labels(), b.get_labels()[:few])
+
+
+# sites such that `few` chains take a lane per label and `many` the thread form
+@pytest.mark.parametrize("L,sites,few,many", [(5, 2000, 5, 7), (6, 2500, 5, 7), (7, 3600, 5, 7), (8, 5000, 5, 7),
+                                              (9, 2400, 5, 6), (9, 6400, 3, 4)])
+@pytest.mark.parametrize("k", [2, 12])
+def test_label_lanes_and_thread_form_draw_the_same_labels(L, sites, few, many, k):
+    _same_first_chains(wl.random_graph(sites, k=k, L=L, seed=L, w_std=0.3), few, many)
