@@ -614,12 +614,15 @@ __device__ __forceinline__ void add_side_chains(const uint32_t (&bits)[CH][Ent<L
     else add_rows<L, LAYOUT, GLOBAL, CH, 0>(bits, t4, tv, 1, acc);
 }
 
-// The same with a test and an add per entry: for the thread form (k_primal) of 13
-// to 15 labels, whose sums spill at 64 registers either way (36,000 sites, 18
-// chains: L = 14 145 us against 159, L = 15 163 against 183; L = 12 and below
-// even, L = 16 238 against 210).
+// The same with a test and an add per entry, for the thread form (k_primal) of 9,
+// 10 and 12 to 15 labels, where the grouped form needs registers the kernel does not
+// have (64; the sums spill from L = 9 on).  us per sweep, single / grouped: random
+// graphs of degree 24, 5 chains, 79,992 edges: L = 9 76 / 78, L = 10 112 / 115, L = 12
+// 170 / 175; a complete graph of 89 sites, 5 chains, L = 12 180 / 195; the primal step
+// of 36,000 lattice sites, 18 chains: L = 14 145 / 159, L = 15 163 / 183.  L = 11 is
+// even (132 / 131), L = 16 better grouped (466 / 381).
 template <int L, int LAYOUT>
-constexpr bool kSingleAdds = LAYOUT == MRF_LAYOUT_PIVOT && L >= 13 && L <= 15;
+constexpr bool kSingleAdds = LAYOUT == MRF_LAYOUT_PIVOT && L >= 9 && L <= 15 && L != 11;
 
 template <int L, int LAYOUT>
 __device__ __forceinline__ void add_side_single(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
