@@ -242,7 +242,26 @@ cudaError_t launch_accumulate(const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_philox_rate(uint64_t threads, int calls, uint32_t* sink, cudaStream_t s);
 cudaError_t launch_log_v(const SweepArgs& a, const double* ut, double* out, cudaStream_t s);
 cudaError_t launch_em(const SweepArgs& a, int layout, const uint8_t* xin, uint8_t* xout, cudaStream_t s);
-cudaError_t launch_sweep_small(const SweepArgs& a, int layout, int n_sweeps, cudaStream_t s);
+// Several plain sweeps of a small model in one launch (k_sweep_resident,
+// k_sweep_small): chains per group, CTAs per group, threads and shared memory of a CTA.
+struct SmallPlan {
+    enum Form : int32_t { kSeparate, kResident, kCluster, kOneCta };
+    Form form;
+    int32_t nc, threads;
+    unsigned size;
+    int64_t smem;
+};
+// Words of a thread's table row in k_sweep_resident: plane words and thresholds of its
+// edge, the weights of its site's first incidences (tables of at most 16 entries); an odd
+// number of 16-byte units, so that rows fall on different banks.
+constexpr int small_row_incidences(int m) { return m <= 16 ? 4 : 0; }
+constexpr int small_row_tau(int m) { return (plane_words(m) + m + 3) / 4 * 4; }
+constexpr int small_row_words(int m) { return ((small_row_tau(m) + small_row_incidences(m) * pad4(m)) / 4 | 1) * 4; }
+// Threads of k_sweep_small's one-CTA form.
+constexpr int small_one_cta_threads(int L) { return L <= 10 ? 1024 : 512; }
+// The plan of a model; may_separate: launches per half-step may be the answer (kSeparate).
+SmallPlan plan_small(const SweepArgs& a, int layout, bool may_separate);
+cudaError_t launch_sweep_small(const SweepArgs& a, int layout, int n_sweeps, const SmallPlan& p, cudaStream_t s);
 cudaError_t launch_mf(const SweepArgs& a, int layout, const float* qin, float* qout, cudaStream_t s);
 cudaError_t launch_marg_layout(const float* in, float* out, int N, int L, int C, bool to_abi, cudaStream_t s);
 // Tensor-core MLP (mlp_tc.cu)

@@ -832,13 +832,15 @@ static bool use_mlp_tc(const mrf_t* h) { return h->opt.mlp_path == 0 && mlp_tc_s
 
 // Small models (at most 2^16 (site, chain) and (edge, chain) items) run several
 // plain sweeps in one launch (k_sweep_resident, k_sweep_small: the additions of
-// k_primal).  The limit is where a launch per half-step wins again: a 12^3
-// lattice, L = 8, 32 chains (165,888 edge items): 208 us per 10 sweeps in separate
-// launches, 382 us in one.  Handles on the edge-partial form keep it for every
+// k_primal).  With more than 200 KB of dual words only where plan_small expects that
+// to be faster than launches per half-step, and never with the CTA schedule, whose
+// additions are in another order.  Handles on the edge-partial form keep it for every
 // sweep, so that a chain does not depend on the sweeps per call.
-static bool small_model(const mrf_t* h) {
+static SmallPlan small_model(const mrf_t* h) {
     const int64_t nv = (int64_t)h->N * h->C, ne = h->E_slots * h->C;
-    return nv <= 65536 && ne <= 65536 && !use_partial(h);
+    const bool few_words = ne * h->W * 4 <= 200 * 1024;
+    if (nv > 65536 || ne > 65536 || use_partial(h) || (!few_words && h->schedule == 2)) return SmallPlan{};
+    return plan_small(make_args(h), h->layout, !few_words);
 }
 
 static SwArgs make_sw_args(const mrf_t* h) {
@@ -1060,11 +1062,14 @@ mrf_status mrf_sweep(mrf_t* h, int32_t n_sweeps, int32_t mode) {
         if (st != MRF_OK) return st;
     }
     // small models: all the sweeps in one launch (launch latency dominates there)
-    if (mode == MRF_MODE_PLAIN && n_sweeps >= 2 && small_model(h)) {
-        const SweepArgs a = make_args(h);
-        MRF_CUDA(h, timed(h, MRF_K_SMALL, [&] { return launch_sweep_small(a, h->layout, n_sweeps, h->stream); }));
-        h->sweep_host += n_sweeps;
-        return MRF_OK;
+    if (mode == MRF_MODE_PLAIN && n_sweeps >= 2) {
+        const SmallPlan plan = small_model(h);
+        if (plan.form != SmallPlan::kSeparate) {
+            const SweepArgs a = make_args(h);
+            MRF_CUDA(h, timed(h, MRF_K_SMALL, [&] { return launch_sweep_small(a, h->layout, n_sweeps, plan, h->stream); }));
+            h->sweep_host += n_sweeps;
+            return MRF_OK;
+        }
     }
     const bool graphs = h->opt.use_graphs && h->stream != nullptr && !h->opt.kernel_timing;
     if (graphs && !h->graph[mode] && n_sweeps > 0) {

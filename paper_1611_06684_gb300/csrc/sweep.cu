@@ -3,6 +3,8 @@
 // of sweep_impl.cuh, instantiated in sweep_la.cu, sweep_lb.cu and sweep_lc.cu.
 #include "common.cuh"
 
+#include <algorithm>
+
 namespace mrfk {
 
 template <int L, int LAYOUT> cudaError_t run_dual(const SweepArgs& a, cudaStream_t s);
@@ -230,13 +232,84 @@ cudaError_t launch_init_labels(const SweepArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-template <int L, int LAYOUT> cudaError_t run_sweep_small(const SweepArgs&, int, cudaStream_t);
+template <int L, int LAYOUT> cudaError_t run_sweep_small(const SweepArgs&, int, const SmallPlan&, cudaStream_t);
 
-cudaError_t launch_sweep_small(const SweepArgs& a, int layout, int n_sweeps, cudaStream_t s) {
+// Estimated us per sweep of each form, the smallest taken.  The forms are bound by
+// latency: rounds of edge items, the chain of additions of a thread's sites (at least
+// the longest incidence list), reading table rows through one SM's L1, and waves of
+// groups (of clusters of eight with one CTA per SM the GPU runs 15 at a time).  The
+// coefficients are fitted to 2,792 models measured in every form: lattices, random,
+// preferential-attachment and complete graphs of 2 to 16 labels, 1 to 64 chains and up
+// to 65,536 edge items; the form taken is within 4 % of the best in 95 % of them and
+// within 17 % in 99 %.  us per sweep, resident / cluster / one CTA / separate launches:
+// 50 x 50 grid, L = 2, one chain 3.3 / 5.9 / 14 / 12; 810 lattice sites, L = 8, 16 chains
+// 26 / 29 / 23 / 14 (waves); 6,498 lattice sites, one chain, L = 2 - / 12 / - / 12, L = 8
+// - / 42 / - / 14; complete graphs of 70 sites, L = 2, one chain 22 / 24 / 13 / 27, and
+// of 20 sites, L = 8, 5 chains 45 / 43 / 13 / 16.
+SmallPlan plan_small(const SweepArgs& a, int layout, bool may_separate) {
+    const auto up = [](int64_t x, int64_t y) { return (x + y - 1) / y; };
+    const int M = a.M, W = a.W;
+    const double mean = 2.0 * (double)a.E / a.N, deg = a.max_deg == 0x7FFFFFFF ? mean : a.max_deg;
+    // chains per group: at most two groups per SM, at least 64 items each
+    const int64_t per_chain = std::max<int64_t>({a.E, a.N, 1});
+    const int64_t nc = std::min<int64_t>(a.C, std::max(up(a.C, 304), up(64, per_chain)));
+    const int64_t items = per_chain * nc, ne = a.E * nc, nv = (int64_t)a.N * nc, groups = up(a.C, nc);
+    SmallPlan best{SmallPlan::kSeparate, 0, 0, 0, 0};
+    double t_best = 1e30;
+    auto offer = [&](SmallPlan::Form form, double t, unsigned size, int64_t threads, int64_t smem) {
+        if (t < t_best) { t_best = t; best = SmallPlan{form, (int32_t)nc, (int32_t)threads, size, smem}; }
+    };
+    // us of `size` CTAs per group, `fit` CTAs per SM: base, per round of edge items, per incidence of a thread's
+    // chain of additions, per thousand incidences of a CTA, and the share that each further CTA on the SM adds
+    auto group_time = [&](unsigned size, int64_t threads, int64_t fit, double base, double round, double add, double read,
+                          double share) {
+        const int64_t T = size * threads;
+        fit = std::max<int64_t>(fit, 1);
+        const int64_t slots = size == 1 ? 152 * fit : (size == 2 ? 76 * fit : (size == 4 ? 36 * fit : 17 * fit - 2));
+        const double chain = std::max(deg, (double)up(nv, T) * mean), inc = (double)nv / size * mean / 1e3;
+        const double per_sm = std::max(1.0, std::min((double)fit, (double)groups * size / 152.0));
+        return (double)up(groups, slots) *
+               (base + round * (double)up(ne, T) + (chain * add + inc * read) * (1.0 + share * (per_sm - 1.0)));
+    };
+    constexpr int64_t kSm = 227 * 1024;                    // shared memory of an SM, 1 KB of it per CTA reserved
+    {   // resident: about 256 threads per CTA (64 and 128 measured the same, 512 and more slower: 100 sweeps of
+        // a 32 x 32 grid 329 us against 300), up to 640 where eight CTAs need them (96 registers per thread)
+        unsigned size = 1;
+        while (size < 8 && items > 256ll * size) size *= 2;
+        const int64_t threads = up(up(items, size), 32) * 32;
+        const int64_t smem = 2 * up(nv, 16) * 16 + up(ne * W, 4) * 16 + threads * small_row_words(M) * 4;
+        if (threads <= 640 && smem <= 200 * 1024) {
+            const bool many = size > 1;
+            offer(SmallPlan::kResident, group_time(size, threads, std::min(65536 / (threads * 96), kSm / (smem + 1024)),
+                  (many ? 1.26 + 0.0059 * M : 0.0) + (M > 16 ? 0.0439 * M : 0.0), 0.105, many ? 0.244 + 0.0263 * M : 0.0955 + 0.0199 * M,
+                  0.0111 * M, 0.125), size, threads, smem);
+        }
+    }
+    {   // cluster: dual words and labels through L2; 64 registers up to 8 labels
+        unsigned size = 2;
+        while (size < 8 && items > 512ll * size) size *= 2;
+        const int fit = a.L <= (layout == MRF_LAYOUT_PIVOT ? 8 : 11) ? 2 : 1;
+        offer(SmallPlan::kCluster, group_time(size, 512, fit, 4.55 + 0.0053 * M, 0.869, 0.216 + 0.0246 * M, 0.0939 * M, 0.0308), size, 512, 0);
+    }
+    {   // one CTA: dual words in shared memory, tables in its L1
+        const int64_t threads = std::min<int64_t>(small_one_cta_threads(a.L), up(items, 32) * 32), smem = ne * W * 4;
+        if (smem <= 200 * 1024)
+            offer(SmallPlan::kOneCta, group_time(1, threads, std::min(65536 / (threads * 64), kSm / (smem + 1024)), 0.292, 2.42,
+                  0.0757 + 0.0104 * M, 0.0954 * M, 0.388), 1, threads, smem);
+    }
+    if (may_separate) {
+        const bool lanes = layout == MRF_LAYOUT_PIVOT && a.C % 32 != 0 && a.L >= 5 && a.L <= 9;
+        const double add = lanes ? 0.142 + 0.0028 * M : (a.C % 32 == 0 ? 0.165 + 0.0028 * M : 0.168 + 0.0119 * M);
+        offer(SmallPlan::kSeparate, 0.9 * (11.7 + deg * add + 0.351e-6 * a.N * a.C * mean * M), 0, 0, 0);   // a tenth in their favour
+    }
+    return best;
+}
+
+cudaError_t launch_sweep_small(const SweepArgs& a, int layout, int n_sweeps, const SmallPlan& p, cudaStream_t s) {
     if (layout == MRF_LAYOUT_PIVOT) {
-        MRF_DISPATCH_L(a.L, return (run_sweep_small<LL, MRF_LAYOUT_PIVOT>(a, n_sweeps, s)));
+        MRF_DISPATCH_L(a.L, return (run_sweep_small<LL, MRF_LAYOUT_PIVOT>(a, n_sweeps, p, s)));
     } else {
-        MRF_DISPATCH_L(a.L, return (run_sweep_small<LL, MRF_LAYOUT_DIAG>(a, n_sweeps, s)));
+        MRF_DISPATCH_L(a.L, return (run_sweep_small<LL, MRF_LAYOUT_DIAG>(a, n_sweeps, p, s)));
     }
     return cudaGetLastError();
 }

@@ -1630,21 +1630,31 @@ __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() { cluster_arrive(); cluster_wait(); }
 
-// Dual words of one (edge, chain), written by another CTA of the cluster (L2) or by this one.
-template <int W, bool L2>
+// Dual words of one (edge, chain), written by a CTA of the cluster (L2).
+template <int W>
 __device__ __forceinline__ void load_words(const uint32_t* th, uint32_t (&bits)[W]) {
     if constexpr (W % 2 == 0) {
 #pragma unroll
         for (int w = 0; w < W; w += 2) {
-            const uint2* p = reinterpret_cast<const uint2*>(th + w);
-            const uint2 q = L2 ? __ldcg(p) : *p;
+            const uint2 q = __ldcg(reinterpret_cast<const uint2*>(th + w));
             bits[w] = q.x;
             bits[w + 1] = q.y;
         }
     } else {
 #pragma unroll
-        for (int w = 0; w < W; ++w) bits[w] = L2 ? __ldcg(th + w) : th[w];
+        for (int w = 0; w < W; ++w) bits[w] = __ldcg(th + w);
     }
+}
+
+// Additions of one incidence in the one-launch kernels: grouped (add_side), or entry
+// by entry where that is faster (PIVOT, single over grouped, median of sites of
+// degree 24 and more: L = 5 1.02, L = 6 0.92 in clusters and 1.07 in one CTA, L = 7
+// 0.83 and 0.90, L = 8 0.80 to 0.89, L = 10 0.83, L = 16 0.82).
+template <int L, int LAYOUT, bool CLUSTER>
+__device__ __forceinline__ void add_side_small(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
+                                               int side, float (&acc)[L]) {
+    if constexpr (LAYOUT == MRF_LAYOUT_PIVOT && L >= (CLUSTER ? 6 : 7)) add_side_single<L, LAYOUT>(bits, tau_e, side, acc);
+    else add_side<L, LAYOUT>(bits, tau_e, side, acc);
 }
 
 // n_sweeps whole plain sweeps of a small model in one launch (sizes where
@@ -1658,12 +1668,17 @@ __device__ __forceinline__ void load_words(const uint32_t* th, uint32_t (&bits)[
 // memory by every thread and advanced by the last cluster to finish.
 // Bound by latency (two barriers and their dependent L2 round trips).  50 x 50
 // Ising grid, 10 chains, 10 sweeps: 990 us in one CTA with all chains, 62 us here.
-// CLUSTER = false: one CTA per group of chains, labels and dual words through
-// its L1 (no barrier's acquire drops the lines of its tables either).
+// CLUSTER = false: one CTA per group of chains, labels through its L1 and dual
+// words in shared memory (no barrier's acquire drops the lines of its tables
+// either); the words of the last sweep are stored.  Up to 10 labels 1,024
+// threads, whose 64 registers hold the sums of 512 threads' 128 nearly as well:
+// 512 threads take 1.1 to 1.4 times as long on 512 to 5,120 items, from L = 11
+// on 0.9 times.
 template <int L, int LAYOUT, bool CLUSTER>
-__global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, FastDiv fdn) {
+__global__ void __launch_bounds__(CLUSTER ? 512 : small_one_cta_threads(L)) k_sweep_small(SweepArgs a, int n_sweeps, FastDiv fdn) {
     using E = Ent<L, LAYOUT>;
     constexpr int W = E::W;
+    extern __shared__ __align__(16) uint32_t s_theta[];    // one CTA: [E][nc][W]
     uint32_t rank = 0, size = 1;
     if (CLUSTER) {
         asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
@@ -1694,8 +1709,14 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
                 for (int w = 0; w < W; ++w) bits[w] = 0;
             }
             uint32_t* out = a.theta + ((int64_t)e * C + c) * W;
+            if (CLUSTER || it + 1 == n_sweeps) {
 #pragma unroll
-            for (int w = 0; w < W; ++w) out[w] = bits[w];
+                for (int w = 0; w < W; ++w) out[w] = bits[w];
+            }
+            if (!CLUSTER) {
+#pragma unroll
+                for (int w = 0; w < W; ++w) s_theta[i * W + w] = bits[w];
+            }
         }
         barrier();
         for (uint32_t i = tid; i < nv; i += T) {
@@ -1714,12 +1735,19 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
 #pragma unroll
                 for (int u = 0; u < B; ++u) code[u] = base + u < p1 ? __ldg(&a.inc[base + u].x) : -1;
 #pragma unroll
-                for (int u = 0; u < B; ++u)
-                    if (code[u] >= 0) load_words<W, CLUSTER>(a.theta + ((int64_t)(code[u] >> 1) * C + c) * W, bits[u]);
+                for (int u = 0; u < B; ++u) {
+                    if (code[u] < 0) continue;
+                    if (CLUSTER) load_words<W>(a.theta + ((int64_t)(code[u] >> 1) * C + c) * W, bits[u]);
+                    else {
+                        const uint32_t* th = s_theta + ((uint32_t)(code[u] >> 1) * nc + (c - c0)) * W;
+#pragma unroll
+                        for (int w = 0; w < W; ++w) bits[u][w] = th[w];
+                    }
+                }
 #pragma unroll
                 for (int u = 0; u < B; ++u) {
                     if (code[u] < 0) continue;
-                    add_side<L, LAYOUT>(bits[u], a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
+                    add_side_small<L, LAYOUT, CLUSTER>(bits[u], a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
                     if (++chunk == 32) {
 #pragma unroll
                         for (int x = 0; x < L; ++x) { two_sum_add(hi[x], lo[x], acc[x]); acc[x] = 0.0f; }
@@ -1772,16 +1800,9 @@ __global__ void __launch_bounds__(512) k_sweep_small(SweepArgs a, int n_sweeps, 
 template <int L, int LAYOUT>
 struct SmallResident {
     using E = Ent<L, LAYOUT>;
-    // words of a thread's table row: plane words and thresholds of its edge, the weights of its site's
-    // first KT incidences (tables of at most 16 entries); an odd number of 16-byte units, so that rows
-    // fall on different banks
-    static constexpr int KT = E::M <= 16 ? 4 : 0;
-    static constexpr int TAU = (E::PW + E::M + 3) / 4 * 4;
-    static constexpr int ROW = ((TAU + KT * E::MP) / 4 | 1) * 4;
-    static int64_t labels(int64_t items) { return (items + 15) / 16 * 16; }
-    static int64_t smem(int64_t site_items, int64_t edge_items, int threads) {
-        return 2 * labels(site_items) + (edge_items * E::W + 3) / 4 * 16 + (int64_t)threads * ROW * 4;
-    }
+    static constexpr int KT = small_row_incidences(E::M);
+    static constexpr int TAU = small_row_tau(E::M);
+    static constexpr int ROW = small_row_words(E::M);
 };
 
 __device__ __forceinline__ uint32_t cluster_address(uint32_t shared_address, uint32_t rank) {
@@ -1903,14 +1924,14 @@ __global__ void __launch_bounds__(640) k_sweep_resident(SweepArgs a, int n_sweep
                 if constexpr (S::KT > 0)
                     add_side<L, LAYOUT, false>(bits, reinterpret_cast<const float*>(s_row + S::TAU + u * E::MP), code[u] & 1, acc);
                 else
-                    add_side<L, LAYOUT>(bits, a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
+                    add_side_small<L, LAYOUT, true>(bits, a.tau + (int64_t)(code[u] >> 1) * E::MP, code[u] & 1, acc);
                 flush();
             }
             for (int u = KI; u < deg; ++u) {
                 const int cd = __ldg(&a.inc[p0 + u].x);
                 uint32_t bits[W];
                 words(cd, bits);
-                add_side<L, LAYOUT>(bits, a.tau + (int64_t)(cd >> 1) * E::MP, cd & 1, acc);
+                add_side_small<L, LAYOUT, true>(bits, a.tau + (int64_t)(cd >> 1) * E::MP, cd & 1, acc);
                 flush();
             }
             float F[L];
@@ -2261,51 +2282,31 @@ cudaError_t run_mf(const SweepArgs& a, const float* qin, float* qout, cudaStream
 }
 
 template <int L, int LAYOUT>
-cudaError_t run_sweep_small(const SweepArgs& a, int n_sweeps, cudaStream_t s) {
-    using S = SmallResident<L, LAYOUT>;
-    // Chains per cluster: at most two clusters per SM, at least 64 items each.  CTAs per cluster: a
-    // power of two, one item per thread and about 256 threads (64 and 128 measured the same, 512 and
-    // 1,024 slower: 100 sweeps of a 32 x 32 Ising grid 329 and 404 us against 300).  Models with more
-    // than 8 x 640 items per cluster, or more than 200 KB of tables per CTA, take k_sweep_small.
-    const int64_t per_chain = std::max<int64_t>(std::max<int64_t>(a.E, a.N), 1);
-    const int64_t nc = std::min<int64_t>(a.C, std::max<int64_t>((a.C + 303) / 304, (64 + per_chain - 1) / per_chain));
-    const int64_t items = per_chain * nc;
-    unsigned size = 1;
-    while (size < 8 && items > 256ll * size) size *= 2;
-    int64_t threads = ((items + size - 1) / size + 31) / 32 * 32;
-    int64_t smem = threads <= 640 ? S::smem(a.N * nc, a.E * nc, (int)threads) : 0;
-    // Sites of many incidences with full tables read most weights from memory in every sweep: one CTA
-    // per group of chains, whose L1 keeps them (complete graphs, 2 chains, us per 10 sweeps, cluster /
-    // one CTA: L = 6, 55 sites 639 / 464, 100 sites 1,113 / 948, 200 sites 1,945 / 2,096; L = 3, 55 sites
-    // 190 / 126; L = 2, 100 sites, 10 chains 335 / 442).
-    const bool one = a.M >= 4 && 2 * a.E >= 24 * (int64_t)a.N && items <= 5120;
-    const bool resident = threads <= 640 && smem <= 200 * 1024 && !one;
-    if (!resident) {
-        size = 1;
-        while (!one && size < 8 && items > 512ll * size) size *= 2;
-        threads = 512;
-        smem = 0;
-    }
+cudaError_t run_sweep_small(const SweepArgs& a, int n_sweeps, const SmallPlan& p, cudaStream_t s) {
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((a.C + nc - 1) / nc) * size);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.gridDim = dim3((unsigned)((a.C + p.nc - 1) / p.nc) * p.size);
+    cfg.blockDim = dim3((unsigned)p.threads);
+    cfg.dynamicSmemBytes = (size_t)p.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = size;
+    attr.val.clusterDim.x = p.size;
     attr.val.clusterDim.y = 1;
     attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = size > 1 ? 1 : 0;
-    if (!resident)
-        return size > 1 ? cudaLaunchKernelEx(&cfg, k_sweep_small<L, LAYOUT, true>, a, n_sweeps, FastDiv::make((uint32_t)nc))
-                        : cudaLaunchKernelEx(&cfg, k_sweep_small<L, LAYOUT, false>, a, n_sweeps, FastDiv::make((uint32_t)nc));
-    if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_sweep_resident<L, LAYOUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaLaunchKernelEx(&cfg, k_sweep_resident<L, LAYOUT>, a, n_sweeps, FastDiv::make((uint32_t)nc));
+    cfg.numAttrs = p.size > 1 ? 1 : 0;
+    const FastDiv fdn = FastDiv::make((uint32_t)p.nc);
+    auto launch = [&](auto kernel) {
+        if (p.smem > 48 * 1024) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaLaunchKernelEx(&cfg, kernel, a, n_sweeps, fdn);
+    };
+    if (p.form == SmallPlan::kResident) return launch(k_sweep_resident<L, LAYOUT>);
+    if (p.form == SmallPlan::kCluster) return launch(k_sweep_small<L, LAYOUT, true>);
+    if (p.form == SmallPlan::kOneCta) return launch(k_sweep_small<L, LAYOUT, false>);
+    return cudaErrorInvalidValue;
 }
 
 template <int L, int LAYOUT>
@@ -2327,8 +2328,8 @@ cudaError_t run_em_pot(const SweepArgs& a, const uint8_t* xin, cudaStream_t s) {
     template cudaError_t run_mf_pot<L, MRF_LAYOUT_DIAG>(const SweepArgs&, const float*, cudaStream_t);  \
     template cudaError_t run_em_pot<L, MRF_LAYOUT_PIVOT>(const SweepArgs&, const uint8_t*, cudaStream_t); \
     template cudaError_t run_em_pot<L, MRF_LAYOUT_DIAG>(const SweepArgs&, const uint8_t*, cudaStream_t);  \
-    template cudaError_t run_sweep_small<L, MRF_LAYOUT_PIVOT>(const SweepArgs&, int, cudaStream_t); \
-    template cudaError_t run_sweep_small<L, MRF_LAYOUT_DIAG>(const SweepArgs&, int, cudaStream_t);  \
+    template cudaError_t run_sweep_small<L, MRF_LAYOUT_PIVOT>(const SweepArgs&, int, const SmallPlan&, cudaStream_t); \
+    template cudaError_t run_sweep_small<L, MRF_LAYOUT_DIAG>(const SweepArgs&, int, const SmallPlan&, cudaStream_t);  \
     template cudaError_t run_em<L, MRF_LAYOUT_PIVOT>(const SweepArgs&, const uint8_t*, uint8_t*, cudaStream_t); \
     template cudaError_t run_em<L, MRF_LAYOUT_DIAG>(const SweepArgs&, const uint8_t*, uint8_t*, cudaStream_t);  \
     template cudaError_t run_mf<L, MRF_LAYOUT_PIVOT>(const SweepArgs&, const float*, float*, cudaStream_t);     \
