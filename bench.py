@@ -1454,6 +1454,7 @@ def main():
     ap.add_argument("--cpu-seconds", type=float, default=10.0, help="time budget of each CPU baseline sample")
     ap.add_argument("--no-configs", action="store_true",
                     help="skip the other workloads' lines (fully connected, batched, learned) of the default run")
+    ap.add_argument("--full-line", action="store_true", help="print every form's kernels and ESS tables on the line")
     args = ap.parse_args()
     args.warmup = max(args.warmup, 3)
     if args.ferro_beta:
@@ -1473,7 +1474,40 @@ def main():
             and args.workload == "potts3d" and not args.scale):
         out["other_configs"] = other_configs(args)
     if rank == 0 and out is not None:
+        if args.impl == "ours" and not args.full_line:
+            print(json.dumps(out), file=sys.stderr)
+            out = compact_line(out)
         print(json.dumps(out))
+
+
+def _short(x):
+    """Numbers to six significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: _short(v) for k, v in x.items()}
+    return x
+
+
+def compact_line(out):
+    """The line's standard keys and one figure per kernel, sweep form and other
+    workload (the full line, with every form's kernels and ESS tables, is 30 KB
+    and more: readers that keep the end of a run's output lost its head)."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else d
+    line = {k: v for k, v in out.items() if k not in ("variants", "other_configs", "roofline", "kernels", "e2e", "cpu_baseline")}
+    line["roofline"] = pick(out["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic", "kernel")
+    line["kernels_ms"] = {k: v["ms_per_launch"] for k, v in out["kernels"].items()}
+    line["variants_ms_per_step"] = {k: v["ms_per_step"] for k, v in out["variants"].items() if "ms_per_step" in v}
+    line["e2e"] = pick(out["e2e"], "value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step")
+    line["cpu_baseline"] = pick(out["cpu_baseline"], "kind", "cores", "sample", "value", "unit")
+    if "other_configs" in out:
+        line["other_configs"] = {
+            name: pick(o, "unavailable") or {"value": o.get("value"), "ms_per_step": o.get("ms_per_step"),
+                                             "e2e": (o.get("e2e") or {}).get("value"),
+                                             "frac": (o.get("roofline") or {}).get("frac")}
+            for name, o in out["other_configs"].items()}
+    return _short(line)
 
 
 def other_configs(args):
@@ -1487,7 +1521,7 @@ def other_configs(args):
             "ba_learned_1e6": ["--workload", "ba_learned", "--steps", "20", "--warmup", "3", "--ess-sweeps", "0"]}
     out = {}
     for name, extra in runs.items():
-        cmd = [sys.executable, os.path.abspath(__file__)] + extra + ["--no-configs", "--seed", str(args.seed),
+        cmd = [sys.executable, os.path.abspath(__file__)] + extra + ["--no-configs", "--full-line", "--seed", str(args.seed),
                                                                      "--cpu-seconds", "5"]
         if args.no_cpu:
             cmd.append("--no-cpu")
