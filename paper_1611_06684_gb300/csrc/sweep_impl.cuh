@@ -2138,14 +2138,16 @@ cudaError_t run_dual(const SweepArgs& a, cudaStream_t s) {
     // few chains and wide tables (two groups per warp): 128 registers and two blocks per SM; at 64
     // registers the 8-word form spills (224 B); with one chain on 25.2 M edges of L = 16 (the
     // 2,000-graph batch's largest class) it measured 5.14 vs 4.12 ms per sweep
-    // groups per warp: NG, or as many as leave four blocks per SM (199,852 edges of L = 2, one chain,
-    // 16 groups per warp are 49 blocks: 33 us, 9 us with one)
-    // (wide tables: one block per SM; 102,060 items of L = 14 in two groups per warp 24 us, in one 27 us)
-    // The variable bound costs up to 9 %, so NG stays where it leaves two blocks per SM.
-    const int64_t per_sm = Ent<L, LAYOUT>::W >= 4 ? 1 : 4;
-    const int ng = n >= 32ll * T::WARPS * T::NG * 152 * 2
-                       ? T::NG
-                       : (int)std::min<int64_t>(T::NG, std::max<int64_t>(1, n / (32 * T::WARPS * 152 * per_sm)));
+    // groups per warp: NG where it leaves two blocks per SM (the variable bound costs up to 9 %), else the
+    // largest power of two that leaves four blocks per SM (199,852 edges of L = 2, one chain: 16 groups per
+    // warp are 49 blocks, 33 us; one group 9 us), two for two and three dual words, one for wide tables.
+    // Other counts leave the last blocks to some SMs: 605,694 items of L = 6, one chain, in 1 / 2 / 3 / 4 / 8
+    // groups 22.4 / 19.7 / 22.8 / 18.9 / 22.5 us; 226,688 items of L = 8, 32 chains, in 1 / 2 / 4 12.4 / 11.4 / 12.4;
+    // 302,400 items in 3 13.8, in 4 12.3; 102,060 items of L = 14 in 1 / 2 27 / 24.
+    const int64_t per_sm = Ent<L, LAYOUT>::W >= 4 ? 1 : (Ent<L, LAYOUT>::W >= 2 ? 2 : 4);
+    int ng = T::NG;
+    if (n < 32ll * T::WARPS * T::NG * 152 * 2)
+        while (ng > 1 && n < 32ll * T::WARPS * ng * 152 * per_sm) ng /= 2;
     const unsigned blocks = blocks_for(n, 32 * ng * T::WARPS);
     if (a.C < 32 && T::NG <= 2) {
         if (ng < T::NG) k_dual<L, LAYOUT, (T::NG <= 2), true><<<blocks, 32 * T::WARPS, 0, s>>>(a, ng);

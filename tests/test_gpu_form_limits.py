@@ -34,3 +34,15 @@ def _same_first_chains(model, few, many, seed=5, sweeps=3):
 @pytest.mark.parametrize("k", [2, 12])
 def test_label_lanes_and_thread_form_draw_the_same_labels(L, sites, few, many, k):
     _same_first_chains(wl.random_graph(sites, k=k, L=L, seed=L, w_std=0.3), few, many)
+
+
+# chains on both sides of the limits of the low-degree form (items, chains) and of the groups per warp of the dual step
+@pytest.mark.parametrize("L,side,few,many", [(2, 28, 14, 18), (3, 28, 14, 18), (4, 28, 14, 18), (5, 40, 4, 6), (6, 52, 7, 9),
+                                             (8, 20, 6, 9), (8, 20, 9, 12), (8, 20, 12, 15), (7, 20, 6, 12), (9, 20, 9, 15)])
+def test_low_degree_and_dual_group_limits_draw_the_same_labels(L, side, few, many):
+    _same_first_chains(wl.potts_grid3d(side, L=L, seed=L), few, many, sweeps=2)
+
+
+@pytest.mark.parametrize("L,side,few,many", [(3, 40, 4, 6), (4, 40, 4, 6), (8, 20, 3, 5)])
+def test_low_degree_form_of_diagonal_tables(L, side, few, many):
+    _same_first_chains(wl.ferro_potts_grid3d(side, L=L, seed=L), few, many, sweeps=2)
