@@ -614,15 +614,18 @@ __device__ __forceinline__ void add_side_chains(const uint32_t (&bits)[CH][Ent<L
     else add_rows<L, LAYOUT, GLOBAL, CH, 0>(bits, t4, tv, 1, acc);
 }
 
-// The same with a test and an add per entry, for the thread form (k_primal) of 9,
-// 10 and 12 to 15 labels, where the grouped form needs registers the kernel does not
-// have (64; the sums spill from L = 9 on).  us per sweep, single / grouped: random
-// graphs of degree 24, 5 chains, 79,992 edges: L = 9 76 / 78, L = 10 112 / 115, L = 12
-// 170 / 175; a complete graph of 89 sites, 5 chains, L = 12 180 / 195; the primal step
-// of 36,000 lattice sites, 18 chains: L = 14 145 / 159, L = 15 163 / 183.  L = 11 is
-// even (132 / 131), L = 16 better grouped (466 / 381).
-template <int L, int LAYOUT>
-constexpr bool kSingleAdds = LAYOUT == MRF_LAYOUT_PIVOT && L >= 9 && L <= 15 && L != 11;
+// The same with a test and an add per entry, for the thread form (k_primal) of 3, 7
+// to 10 and 12 to 15 labels: the grouped form holds a block's weights and predicates
+// at once, and at 64 registers its sums spill from L = 9 on.  us per sweep, single /
+// grouped: random graphs of degree 24, 5 chains, 79,992 edges: L = 9 76 / 78, L = 10
+// 112 / 115, L = 12 170 / 175; a complete graph of 89 sites, 5 chains, L = 12 180 / 195;
+// the primal step of two million lattice items: L = 3 0.85 to 1.0 times the grouped
+// form's time, L = 7 0.93 to 0.97, L = 8 0.92 to 1.0; 36,000 sites, 18 chains: L = 14
+// 145 / 159, L = 15 163 / 183.  L = 6 and 11 are even, L = 2, 4, 5 up to 1.1 and L = 16
+// (466 / 381) better grouped.  The fused form has 128 registers: 13 to 15 labels only.
+template <int L, int LAYOUT, bool FUSED>
+constexpr bool kSingleAdds = LAYOUT == MRF_LAYOUT_PIVOT &&
+                             (FUSED ? L >= 13 && L <= 15 : L == 3 || (L >= 7 && L <= 15 && L != 11));
 
 template <int L, int LAYOUT>
 __device__ __forceinline__ void add_side_single(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
@@ -733,7 +736,7 @@ __global__ void __launch_bounds__(256, FUSED ? 2 : 4) k_primal(SweepArgs a) {
 #pragma unroll
         for (int u = 0; u < B; ++u) {
             if (ic[u].x < 0) continue;
-            if constexpr (kSingleAdds<L, LAYOUT>) add_side_single<L, LAYOUT>(bits[u], a.tau + (ic[u].x >> 1) * (int64_t)E::MP, ic[u].x & 1, acc);
+            if constexpr (kSingleAdds<L, LAYOUT, FUSED>) add_side_single<L, LAYOUT>(bits[u], a.tau + (ic[u].x >> 1) * (int64_t)E::MP, ic[u].x & 1, acc);
             else add_side<L, LAYOUT>(bits[u], a.tau + (ic[u].x >> 1) * (int64_t)E::MP, ic[u].x & 1, acc);
             if (++chunk == 32) {
 #pragma unroll
@@ -765,8 +768,9 @@ __global__ void __launch_bounds__(256, FUSED ? 2 : 4) k_primal(SweepArgs a) {
 // Thread form for sites of at most KB incidences: every incidence code, then
 // every dual word of the site is loaded before any is used (two dependent loads
 // where batches of four made four), and no two-sum pair is kept, since no sum
-// reaches 32 incidences.  Keeps k_primal's order of additions.  151,951 sites of a
-// lattice, L = 5, 24 chains: 120 -> 101 us.
+// reaches 32 incidences.  Keeps k_primal's order of additions (entry by entry: 0.92
+// to 0.98 of the grouped form's time at L = 5).  151,951 sites of a lattice, L = 5,
+// 24 chains: 120 -> 101 us with grouped additions, 0.95 of that with single ones.
 template <int L, int LAYOUT, bool POT = false>
 __global__ void __launch_bounds__(256, 4) k_primal_low(SweepArgs a) {
     using E = Ent<L, LAYOUT>;
@@ -798,8 +802,11 @@ __global__ void __launch_bounds__(256, 4) k_primal_low(SweepArgs a) {
     for (int x = 0; x < L; ++x) acc[x] = 0.0f;
 #pragma unroll
     for (int u = 0; u < KB; ++u)
-        if (code[u] >= 0)
-            add_side<L, LAYOUT>(bits[u], a.tau + (uint64_t)((uint32_t)code[u] >> 1) * E::MP, code[u] & 1, acc);
+        if (code[u] >= 0) {
+            const float* tau = a.tau + (uint64_t)((uint32_t)code[u] >> 1) * E::MP;
+            if constexpr (LAYOUT == MRF_LAYOUT_PIVOT) add_side_single<L, LAYOUT>(bits[u], tau, code[u] & 1, acc);
+            else add_side<L, LAYOUT>(bits[u], tau, code[u] & 1, acc);
+        }
     float F[L];
     const float* uf = a.utf + (int64_t)v * L;
 #pragma unroll
@@ -2210,6 +2217,21 @@ cudaError_t run_primal_warps(const SweepArgs& a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+// Where k_primal_low beats the thread form (time over the thread form's, 100,000 to two
+// million items of 2-d and 3-d lattices, 1 to 40 chains): L = 9 0.89 to 1.0, at 20,000
+// items up to 1.17; L = 8 1.0 to 1.2, L = 7 0.91 to 1.05; L = 6 0.88 to 1.02 from a million items, up to 1.18 below; L = 5
+// 0.83 to 1.0 from 300,000, up to 1.04 below; L = 2 to 4 only with many chains, whose
+// lanes share the codes and weights, and six incidences: 0.86 to 1.0, else up to 1.2.
+// Diagonal tables 0.77 to 1.0, L = 3 and 4 below 300,000 items up to 1.1.
+template <int L, int LAYOUT>
+bool low_form_wins(const SweepArgs& a, int64_t n) {
+    constexpr int64_t kSome = 300000, kMany = 1 << 20;
+    if (LAYOUT == MRF_LAYOUT_DIAG) return L >= 8 || n >= kSome;
+    if (L >= 7) return L == 9 && n >= 65536;
+    if (L >= 5) return n >= (L == 6 ? kMany : kSome);
+    return n >= kSome && a.C >= 16 && a.max_deg >= 5;
+}
+
 // Thread or warp form of the plain primal step or its potentials.  A graph
 // with hubs leaves them to a second launch; where the largest degree may
 // change between launches (a batch's edit queue) there is none.
@@ -2246,7 +2268,7 @@ cudaError_t run_field(const SweepArgs& args, cudaStream_t s) {
     } else {
         bool low = false;
         if constexpr (Ent<L, LAYOUT>::W <= 2) {
-            low = a.max_deg <= 8;
+            low = a.max_deg <= 8 && low_form_wins<L, LAYOUT>(a, n);
             if (low) k_primal_low<L, LAYOUT, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
         }
         if (!low) k_primal<L, LAYOUT, false, POT><<<blocks_for(n, 256), 256, 0, s>>>(a);
