@@ -1674,16 +1674,19 @@ void free_queue(mrf_batch_t* b, bool keep_mirror = true) {
 }
 
 // Runs fn(k, stream) for every class: one after another on the batch's stream
-// or, while that stream is captured, each class in a branch of its own, so that
-// the classes' kernels, too small to fill the GPU in a batch of a few dozen
-// graphs, run beside each other (40 graphs, edit and 10 sweeps: the kernels'
-// times sum to 4.4 ms, the round takes 2.6 ms).  The classes share
-// no buffer.  enqueue_sweep follows the class handle's stream, which is the
-// branch's while fn runs.
+// or, where `branches` is set while that stream is captured, each class in a branch of
+// its own, so that the classes' kernels, too small to fill the GPU in a batch of a few
+// dozen graphs, run beside each other (40 graphs, edit and 10 sweeps: the kernels'
+// times sum to 4.4 ms, the round takes 2.6 ms).  enqueue_sweep follows the class
+// handle's stream, which is the branch's while fn runs.  The classes share three
+// buffers, all of the edit queue: the status word, whose fatal bits are final before
+// the fork (a check inside a branch must not set one, since the other branches read it
+// unordered; k_q_place's repeats a check made before and cannot fire), the result slots, of which each class writes its own additions', and
+// the CSR's count of long lists, which a round does not read.
 template <class Fn>
-mrf_status for_classes(mrf_batch_t* b, bool capturing, Fn fn) {
+mrf_status for_classes(mrf_batch_t* b, bool branches, Fn fn) {
     const int K = (int)b->h.size();
-    if (!capturing || K < 2) {
+    if (!branches || K < 2) {
         for (int k = 0; k < K; ++k) {
             const mrf_status st = fn(k, b->stream);
             if (st != MRF_OK) return st;
@@ -2054,14 +2057,22 @@ QArgs make_qargs(const mrf_batch_t* b) {
 }
 
 // The kernels of one round on the batch's stream (captured or launched): the
-// edit's route and checks, then per class the edit and the sweeps.
+// edit's route and checks, then per class the edit and the sweeps.  A captured round
+// of classes that fill the GPU on their own runs them one after another: branches that
+// drift apart over the sweeps take the L2 from each other.  Round of an edit and 10
+// sweeps, branches / one after another, by the classes' dual words in millions: 1.5
+// 1.6 / 2.4 ms, 5.3 5.5 / 6.0, 9.8 7.4 / 8.4, 13.6 10.6 / 10.9, 26 22.1 / 19.1, 104
+// 42.4 / 39.1; 2,000 graphs 319 / 186 ms.
 mrf_status enqueue_round(mrf_batch_t* b, int n_sweeps, int mode, bool capturing) {
+    constexpr int64_t kBranchWords = 1 << 24;
+    int64_t words = 0;
+    for (const mrf_t* h : b->h) words += h->E_slots * h->C * h->W;
     const QArgs q = make_qargs(b);
     cudaError_t e = cudaMemsetAsync(b->dq_status, 0, sizeof(uint32_t), b->stream);
     if (e == cudaSuccess) e = launch_queue_route(q, b->stream);
     auto failed = [&] { cudaGetLastError(); return bfail(b, MRF_ECUDA, std::string("round launch: ") + cudaGetErrorString(e)); };
     if (e != cudaSuccess) return failed();
-    mrf_status st = for_classes(b, capturing, [&](int k, cudaStream_t s) {
+    mrf_status st = for_classes(b, capturing && words <= kBranchWords, [&](int k, cudaStream_t s) {
         mrf_t* h = b->h[k];
         const QClass& c = b->qc[k];
         e = launch_queue_apply(q, c, s);
