@@ -1,5 +1,5 @@
-// Device-side CSR incidence build, used after edits so that a dynamic model
-// never round-trips its edge list through the host.  The result is identical
+// Device-side CSR incidence build, used when factors are set and after edits, so that a
+// dynamic model never round-trips its edge list through the host.  The result is identical
 // to the host build: within a site, incidences in increasing edge slot order
 // (a site is never both ends of one edge), code = slot * 2 + side.
 //   1. degree of every site over live edges (atomics)
