@@ -600,8 +600,10 @@ mrf_status mrf_set_factors(mrf_t* h, const float* unary_log, int64_t n_edges, co
     MRF_CUDA(h, to_device(h->d_unary, unary, (int64_t)N * L, MRF_PTR_DEVICE, s));
     MRF_CUDA(h, to_device(h->d_src, src, n_edges, ptr_kind, s));
     MRF_CUDA(h, to_device(h->d_dst, dst, n_edges, ptr_kind, s));
-    // incidence lists on the device (sites of more than 512 incidences sorted by a CTA each; on the host
-    // if one is too long for that)
+    // incidence lists on the device (sites of more than 32 incidences sorted by a CTA each, since a thread's
+    // insertion sort is quadratic: a preferential-attachment graph of 20,000 sites took 4.6 ms with a limit of
+    // 512 and 1.9 ms on the host; on the host if one is too long for that)
+    constexpr int kCsrThreadSort = 32;
     if (!h->d_inc_ptr) MRF_CUDA(h, dalloc(h->d_inc_ptr, (size_t)N + 1));
     if (2 * n_edges > h->inc_cap || !h->d_inc) {
         MRF_CUDA(h, dalloc(h->d_inc, std::max<size_t>(2 * E, 1)));
@@ -614,8 +616,8 @@ mrf_status mrf_set_factors(mrf_t* h, const float* unary_log, int64_t n_edges, co
     MRF_CUDA(h, init_csr_sort_long());
     MRF_CUDA(h, cudaMemsetAsync(h->d_flag, 0, sizeof(flag), s));
     MRF_CUDA(h, build_csr_device(h->d_src, h->d_dst, n_edges, N, h->d_inc_ptr, h->d_inc, h->d_csr_work, h->d_csr_sums,
-                                 h->d_flag, 512, s));
-    MRF_CUDA(h, launch_csr_sort_long(h->d_inc_ptr, h->d_inc, N, 512, reinterpret_cast<uint32_t*>(h->d_flag + 1), s));
+                                 h->d_flag, kCsrThreadSort, s));
+    MRF_CUDA(h, launch_csr_sort_long(h->d_inc_ptr, h->d_inc, N, kCsrThreadSort, reinterpret_cast<uint32_t*>(h->d_flag + 1), s));
     MRF_CUDA(h, launch_max_degree(h->d_inc_ptr, N, reinterpret_cast<unsigned*>(h->d_flag + 2), s));
     DecompArgs d{};
     d.L = L; d.M = h->M; d.layout = h->layout; d.n = n_edges; d.slots = nullptr; d.first_slot = 0;

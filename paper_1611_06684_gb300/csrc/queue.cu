@@ -321,10 +321,11 @@ __global__ void __launch_bounds__(256) k_csr_sort_long(const int64_t* __restrict
     extern __shared__ int2 s_inc[];
     __shared__ int s_list[256];
     __shared__ int s_n;
-    for (int64_t v0 = (int64_t)blockIdx.x * 256; v0 < N; v0 += (int64_t)gridDim.x * 256) {
+    // a block's 256 sites are gridDim.x apart: long lists come in runs (the first sites of a preferential-attachment graph)
+    for (int64_t v0 = blockIdx.x; v0 < N; v0 += (int64_t)gridDim.x * 256) {
         if (threadIdx.x == 0) s_n = 0;
         __syncthreads();
-        const int64_t v = v0 + threadIdx.x;
+        const int64_t v = v0 + (int64_t)threadIdx.x * gridDim.x;
         if (v < N && ptr[v + 1] - ptr[v] > min_deg) s_list[atomicAdd(&s_n, 1)] = (int)v;
         __syncthreads();
         const int n = s_n;
@@ -336,7 +337,7 @@ __global__ void __launch_bounds__(256) k_csr_sort_long(const int64_t* __restrict
                 if (threadIdx.x == 0) atomicOr(status, kQUnsorted);
                 continue;
             }
-            int P = 1024;                                  // the next power of two
+            int P = 64;                                    // the next power of two
             while (P < d) P *= 2;
             if (P <= cap) {                                // bitonic sort, padded with the largest code
                 for (int i = threadIdx.x; i < P; i += 256) s_inc[i] = i < d ? inc[p0 + i] : make_int2(0x7FFFFFFF, 0);

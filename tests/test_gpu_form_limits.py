@@ -46,3 +46,37 @@ def test_low_degree_and_dual_group_limits_draw_the_same_labels(L, side, few, man
 @pytest.mark.parametrize("L,side,few,many", [(3, 40, 4, 6), (4, 40, 4, 6), (8, 20, 3, 5)])
 def test_low_degree_form_of_diagonal_tables(L, side, few, many):
     _same_first_chains(wl.ferro_potts_grid3d(side, L=L, seed=L), few, many, sweeps=2)
+
+
+# largest lists of 119, 199 and 299 incidences: on both sides of the hub launch's limits for up to 32 chains and more
+@pytest.mark.parametrize("sites,few,many", [(120, 3, 40), (200, 3, 40), (200, 32, 33), (300, 3, 40)])
+def test_hub_limits_draw_the_same_labels(sites, few, many):
+    _same_first_chains(wl.dense_potts(sites, L=4, seed=sites), few, many, sweeps=2)
+
+
+@pytest.mark.parametrize("device", [False, True])
+def test_incidence_lists_of_every_length_are_in_order(device):
+    # lists of 0 to 700 incidences, long ones next to each other: folded unaries (summed in list order) and
+    # labels equal those of a handle whose lists were rebuilt by an edit that changes nothing
+    import torch
+    from paper_1611_06684_gb300 import mrf as M
+    rng = np.random.default_rng(3)
+    hub = rng.integers(0, 40, 6000)
+    other = 40 + rng.integers(0, 900, 6000)
+    hub[:700], other[:700] = 7, 40 + np.arange(700)
+    hub[700:733], other[700:733] = 990, 1000 + np.arange(33)           # 33 and 32: the sorts' border
+    hub[733:765], other[733:765] = 991, 1000 + np.arange(32)
+    m = wl.Model(1100, 3, rng.normal(size=(1100, 3)).astype(np.float32), hub.astype(np.int32), other.astype(np.int32),
+                 rng.normal(0, 0.1, (6000, 3, 3)).astype(np.float32))
+    h, e = (M.MRF(m.n_vars, 3, 5, seed=2, schedule=1) for _ in range(2))
+    arrays = (m.unary, m.src, m.dst, m.pair)
+    h.set_factors(*(tuple(torch.from_numpy(x).cuda() for x in arrays) if device else arrays))
+    e.set_factors(*arrays)
+    e.edit_factors(np.array([11]), m.src[11:12], m.dst[11:12], m.pair[11:12])
+    for x, y in zip(h.debug_tables(), e.debug_tables()):
+        assert np.array_equal(x, y)
+    fold = m.unary.astype(np.float64)
+    assert not np.array_equal(h.debug_tables()[2], fold)
+    for g in (h, e):
+        g.sweep(3)
+    assert np.array_equal(h.get_labels(), e.get_labels())
