@@ -622,10 +622,11 @@ __device__ __forceinline__ void add_side_chains(const uint32_t (&bits)[CH][Ent<L
 // the primal step of two million lattice items: L = 3 0.85 to 1.0 times the grouped
 // form's time, L = 7 0.93 to 0.97, L = 8 0.92 to 1.0; 36,000 sites, 18 chains: L = 14
 // 145 / 159, L = 15 163 / 183.  L = 6 and 11 are even, L = 2, 4, 5 up to 1.1 and L = 16
-// (466 / 381) better grouped.  The fused form has 128 registers: 13 to 15 labels only.
+// (466 / 381) better grouped.  The fused form: from 8 labels on (76,000 lattice sites, 2
+// chains: L = 8 57 / 63, L = 10 90 / 102, L = 12 122 / 135, L = 16 256 / 284).
 template <int L, int LAYOUT, bool FUSED>
 constexpr bool kSingleAdds = LAYOUT == MRF_LAYOUT_PIVOT &&
-                             (FUSED ? L >= 13 && L <= 15 : L == 3 || (L >= 7 && L <= 15 && L != 11));
+                             (FUSED ? L >= 8 : L == 3 || (L >= 7 && L <= 15 && L != 11));
 
 template <int L, int LAYOUT>
 __device__ __forceinline__ void add_side_single(const uint32_t (&bits)[Ent<L, LAYOUT>::W], const float* __restrict__ tau_e,
