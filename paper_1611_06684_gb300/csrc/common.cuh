@@ -230,11 +230,16 @@ cudaError_t launch_primal(const SweepArgs& a, int layout, int schedule, cudaStre
 // Plain sweep in the edge-partial form (few chains, more than 16 entries per
 // edge), after the dual step: step 0 the per-edge partial fields, step 1 the labels.
 cudaError_t launch_sweep_partial(const SweepArgs& a, int layout, int step, cudaStream_t s);
-// Sites of more incidences than this are summed by a CTA each (k_primal_hub).
+// Sites of more than kHubDegree incidences are summed by a CTA each (k_primal_hub).
 // Preferential attachment, us per launch with a limit of 64 / 128 / 256 / none:
 // 50,000 sites, 32 chains 113 / 103 / 125 / 351; 10 chains 87 / 84 / 112 / 412;
 // 5,000 sites, 64 chains 45 / 59 / 90 / 95.
 constexpr int kHubDegree = 96;
+// ... where the largest list is long enough to pay for that launch (with hubs / without,
+// L = 8 diagonal): largest list 97 C = 32 42 / 29, 128 46 / 37, 155 46 / 43, 169 46 / 50,
+// 245 48 / 64; 96 chains, three groups of 32 in a hub's CTA, 169 60 / 49, 245 66 / 66,
+// 289 70 / 79.
+constexpr int hub_min_degree(int C) { return C <= 32 ? 160 : 240; }
 constexpr int kPartialMaxChains = 4;
 constexpr int kPartialMinEntries = 100;
 cudaError_t launch_fused(const SweepArgs& a, int layout, int schedule, cudaStream_t s);

@@ -2241,7 +2241,7 @@ cudaError_t run_field(const SweepArgs& args, cudaStream_t s) {
     const int64_t n = (int64_t)args.N * args.C;
     if (n <= 0) return cudaSuccess;
     SweepArgs a = args;
-    const bool hubs = a.max_deg > kHubDegree && a.max_deg != 0x7FFFFFFF;
+    const bool hubs = a.max_deg > hub_min_degree(a.C) && a.max_deg != 0x7FFFFFFF;
     if (hubs) a.hub_deg = kHubDegree;
     cudaError_t e = cudaSuccess;
     bool labels = false;

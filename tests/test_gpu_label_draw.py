@@ -37,7 +37,7 @@ FORMS = {
     "low": (lambda: wl.potts_grid3d(6, 5, 3, L=4, seed=5), 5, 1),
     "thread": (lambda: wl.tiny_random(60, 4, 400, w_std=0.4, seed=6), 5, 1),
     "label_lanes": (lambda: wl.potts_grid3d(6, 5, 3, L=8, seed=7), 5, 1),
-    "hub": (lambda: _star(131, 3, 8), 5, 1),
+    "hub": (lambda: _star(301, 3, 8), 5, 1),
     "cta": (lambda: wl.dense_potts(60, L=4, seed=9), 16, 2),
     "partial": (lambda: wl.random_graph(60, k=2, L=16, seed=10, w_std=0.3), 2, 1),
 }
