@@ -230,16 +230,24 @@ cudaError_t launch_primal(const SweepArgs& a, int layout, int schedule, cudaStre
 // Plain sweep in the edge-partial form (few chains, more than 16 entries per
 // edge), after the dual step: step 0 the per-edge partial fields, step 1 the labels.
 cudaError_t launch_sweep_partial(const SweepArgs& a, int layout, int step, cudaStream_t s);
-// Sites of more than kHubDegree incidences are summed by a CTA each (k_primal_hub).
+// Sites of more than hub_degree incidences are summed by a CTA each (k_primal_hub).
 // Preferential attachment, us per launch with a limit of 64 / 128 / 256 / none:
 // 50,000 sites, 32 chains 113 / 103 / 125 / 351; 10 chains 87 / 84 / 112 / 412;
 // 5,000 sites, 64 chains 45 / 59 / 90 / 95.
-constexpr int kHubDegree = 96;
+// From two million (site, chain) items on the other sites' work hides longer lists (limit 96 / 192;
+// L = 4): 200,000 sites, 10 chains 190 / 163, 64 chains 642 / 607; 10^6 sites, 4 chains 737 / 472;
+// below it 100,000 sites, one chain, L = 8 88 / 97; 50,000 sites, 10 chains, L = 12 87 / 107.
+constexpr int hub_degree(int64_t items) { return items < 2000000 ? 96 : 192; }
 // ... where the largest list is long enough to pay for that launch (with hubs / without,
 // L = 8 diagonal): largest list 97 C = 32 42 / 29, 128 46 / 37, 155 46 / 43, 169 46 / 50,
-// 245 48 / 64; 96 chains, three groups of 32 in a hub's CTA, 169 60 / 49, 245 66 / 66,
-// 289 70 / 79.
+// 245 48 / 64; 96 chains 169 60 / 49, 245 66 / 66, 289 70 / 79.
 constexpr int hub_min_degree(int C) { return C <= 32 ? 160 : 240; }
+// ... and where the other sites' (incidence, chain) additions do not hide the longest list: 200
+// of them take 1 ns, an incidence of one list 0.4 us, so they meet at 80,000 additions per
+// incidence of the longest list.  With hubs / without, L = 4: 200,000 sites, 64 chains (76,000)
+// 607 / 687 us, 96 chains (114,000) 872 / 804, 160 chains (190,000) 1,386 / 1,304; 10^6 sites, 32
+// chains (86,000) 1,687 / 1,558; L = 2, 3 edges per new site, 10^6 sites, 32 chains (52,000) 986 / 1,488.
+constexpr int64_t kHubHidden = 80000;
 constexpr int kPartialMaxChains = 4;
 constexpr int kPartialMinEntries = 100;
 cudaError_t launch_fused(const SweepArgs& a, int layout, int schedule, cudaStream_t s);

@@ -54,6 +54,12 @@ def test_hub_limits_draw_the_same_labels(sites, few, many):
     _same_first_chains(wl.dense_potts(sites, L=4, seed=sites), few, many, sweeps=2)
 
 
+# a CTA's hubs from 97 incidences on, from 193 on with two million items, no hub launch with many chains
+@pytest.mark.parametrize("sites,few,many", [(20000, 3, 96), (40000, 3, 64), (20000, 3, 320), (20000, 32, 330)])
+def test_hub_rules_of_large_models_draw_the_same_labels(sites, few, many):
+    _same_first_chains(wl.ba_potts(sites, m=5, L=4, seed=sites), few, many, sweeps=2)
+
+
 @pytest.mark.parametrize("device", [False, True])
 def test_incidence_lists_of_every_length_are_in_order(device):
     # lists of 0 to 700 incidences, long ones next to each other: folded unaries (summed in list order) and
