@@ -138,8 +138,8 @@ mrf_status mrf_edit_factors(mrf_t* h, int64_t n_remove, const int64_t* edge_ids,
 /* Run n_sweeps sweeps (Section 5.1 or 5.4) and accumulate label counts for
  * sweeps with index >= burn-in.  Asynchronous on the handle's stream.  Plain
  * sweeps of a small model (at most 2^16 site x chain and edge x chain items)
- * with n_sweeps >= 2 run in one launch (the same chain, bit for bit, as one
- * sweep at a time).
+ * with n_sweeps >= 2 run in one launch where that is faster (always with up to
+ * 200 KB of dual words; the same chain, bit for bit, as one sweep at a time).
  *
  * MRF_MODE_SW (Section 4.3): every table is read as c + f(x_s) + g(x_t) +
  * l_{x_s} [x_s = x_t] with f, g folded into the unaries -- Potts-type tables
